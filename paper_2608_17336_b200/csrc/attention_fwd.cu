@@ -24,6 +24,8 @@
 #include <cuda.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx_sm100.cuh"
 #include "quant8.cuh"
@@ -50,6 +52,7 @@ constexpr int kRegsSoftmaxOtf = 96, kRegsOtherOtf = 48;
 static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + (kThreads - kSoftmaxWarps * 32) * kRegsOther <= kThreads * kLaunchRegs, "setmaxnreg split");
 static_assert(kSoftmaxWarps * 32 * kRegsSoftmaxOtf + (kThreadsOtf - kSoftmaxWarps * 32) * kRegsOtherOtf <= kThreadsOtf * kLaunchRegsOtf, "setmaxnreg split");
 constexpr uint32_t kQuantBar = 9;         // named barrier of the quantiser warps
+constexpr int kSms = 148;          // streaming multiprocessors of a B200
 constexpr int kMaxHeadGroup = 8;   // (batch, head) rows whose CTAs are interleaved in the grid order, at most
 constexpr int kRing = 8;
 constexpr int kBundles = 4;        // operand bundles in flight at most (each has a "landed" and a "consumed" barrier)
@@ -74,8 +77,19 @@ enum Role : int { kRoleSoftmaxA = 0, kRoleSoftmaxB = 1, kRoleProducer = 2, kRole
 enum Bar : int { kBarQ = 0, kBarRingFull = 1, kBarRingEmpty = 2, kBarS = 3, kBarP = 4, kBarO = 5, kBarDrain = 6, kBarPV = 7,
                  kBarRaw = 8, kBarQ8 = 9 };
 
-template <int D, int T>
+// D: head dimension.  A "tile" of this file is 128 queries x 128 keys (what one accumulator holds) for both head
+// dimensions.  With D = 128 it is one routing tile.  With D = 64 the routing tiles are 64 x 64 and a tile carries 2 x 2
+// of them (kSub): its two row halves (tensor-memory lanes 0-63 / 64-127) and its two key halves have routes, scales and
+// causal limits of their own; where the two row halves' routes differ both products are issued, each with the other
+// half's accumulator lanes switched off.  D = 64 is bound by the exponentials (512 clk of the special-function unit per
+// 128 x 64 scores against 350-450 of MMAs).  One 64-row routing tile per accumulator, which this replaced, left half of
+// the lanes, and so half of both, to rows that do not exist: quantise + pack + attend over 4 x 2000 tokens, 32 / 8
+// heads, went from 371 to 198 us.
+template <int D>
 struct Cfg {
+    static constexpr int T = 128;
+    static constexpr bool kSub = D == 64;
+    static constexpr int kRT = kSub ? 64 : 128;       // rows / keys of a routing tile
     static constexpr int kM = 128;                    // rows of one MMA / TMEM tile
     static constexpr int kChunk = T * 128;            // ring chunk: T rows of 128 bytes
     static constexpr int kHalves = D / 64;            // 64-element column slabs of an FP16 tile
@@ -88,7 +102,7 @@ struct Cfg {
     static constexpr uint32_t kI8Sbo = 8u * D;
     static constexpr int kSCols = T;
     static constexpr int kOCols = D;
-    static constexpr int kTmemCols = 2 * (kSCols + kOCols);
+    static constexpr int kTmemCols = 512;             // 2 * (kSCols + kOCols), rounded up to a power of two
     static constexpr int kOffQ16 = 0;
     static constexpr int kOffQ8 = 2 * kQ16Tile;
     static constexpr int kOffRing = kOffQ8 + 2 * kQ8Tile;
@@ -100,7 +114,7 @@ struct Cfg {
     static constexpr int kSmemBytes = kOffWords + kMaxTiles / 2;   // 4-bit schedule entries
     static constexpr int kSmemAlloc = kSmemBytes + 1024;           // slack to align the base
     static_assert(kK8Bytes <= kChunk, "INT8 key tile must fit one ring chunk");
-    static_assert(kTmemCols == 256 || kTmemCols == 512, "TMEM allocation must be a power of two");
+    static_assert(2 * (kSCols + kOCols) <= kTmemCols, "tensor memory");
     static_assert(kSmemAlloc <= 232448, "exceeds the 227 KB shared memory of a CTA");
     static_assert(T % 32 == 0 && D % 64 == 0, "tile shape");
 };
@@ -113,6 +127,7 @@ struct Params {
     int test_drop_bundle;              // testing aid: the producer leaves out the copies of this operand bundle (-1: none)
     int head_group;               // (batch, head) rows interleaved in the grid order (>= 1)
     int has_int8;                 // INT8 operands present
+    int solo;                     // 1: one tile per CTA (small grids), 0: two
     float scale_log2;             // softmax scale * log2(e)
     const float* q_scale;         // [B,Hq,T_m]; variable-length batch: [sum T_m, Hq]
     const float* k_scale;         // [B,Hk,T_n]; variable-length batch: [sum T_n, Hk]
@@ -192,12 +207,17 @@ struct Ring {
 // DBG: the instance that can write the raw accumulators of requested tiles (every step then takes the generic form).
 // A kernel of its own, because every instruction in the softmax warps' loop that is not executed still costs: the loop
 // of the other instances is ~1 % faster without that code in it.
-template <int D, int T, bool VL, bool OTF, bool VS = false, bool DBG = false>
+// KH (head dimension 64): quantisation blocks of K of half a routing tile, i.e. two scales per step.  (Head dimension
+// 128 has one scale per step either way and takes both at run time.)
+template <int D, bool VL, bool OTF, bool VS = false, bool DBG = false, bool KH = false>
 __global__ void __launch_bounds__(OTF ? kThreadsOtf : kThreads, 1)
 attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                  const __grid_constant__ CUtensorMap tm_k16, const __grid_constant__ CUtensorMap tm_v16,
                  const __grid_constant__ CUtensorMap tm_q8, const __grid_constant__ CUtensorMap tm_k8) {
-    using C = Cfg<D, T>;
+    using C = Cfg<D>;
+    constexpr int T = C::T;
+    constexpr bool SUB = C::kSub;
+    static_assert(!KH || SUB, "two scales per step only with 64-key routing tiles");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = ptx::smem_u32(smem);
@@ -213,18 +233,20 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     // b: batch coordinate of the tensor maps; seq: sequence index (== b for a dense batch);
     // tok0 / len: first token and length of the sequence; row0: its first row among the mask rows
     // and scale blocks; m, n below count tiles inside the sequence.
-    int b, hq, pr, seq, tok0 = 0, len = prm.L, row0 = VL ? 0 : prm.kv_off, n_rows = prm.T_m;
+    int b, hq, pr, seq, tok0 = 0, len = prm.L, row0 = VL ? 0 : prm.kv_off, n_rows = prm.T_m;   // (rows: of routing tiles)
     int kblk0 = 0, n_kblk = prm.ks_blocks;   // first quantisation block of K of this sequence and their number
     // Order of the grid: (batch, head) rows in groups of head_group; inside a group the longest work items
     // first, and the heads of the group side by side for each item.  The host sizes the group so that its
     // K/V fits in L2 while its CTAs run; the grid then ends with the shortest items of the last group instead
     // of with the long items of the last head, and the SMs finish close together.
+    // With `solo` two adjacent CTAs take the two tiles of a pair (the longer one first).
     const int kHeadGroup = prm.head_group;
+    const int blk = static_cast<int>(blockIdx.x) >> prm.solo;
     if constexpr (!VL) {
-        const int n_pairs = (prm.T_m + 1) >> 1;
+        const int n_pairs = SUB ? (prm.T_m + 3) >> 2 : (prm.T_m + 1) >> 1;
         const int n_bh = prm.B * prm.Hq;
-        const int grp = blockIdx.x / (kHeadGroup * n_pairs);
-        const int in_grp = blockIdx.x - grp * (kHeadGroup * n_pairs);
+        const int grp = blk / (kHeadGroup * n_pairs);
+        const int in_grp = blk - grp * (kHeadGroup * n_pairs);
         const int g_heads = min(kHeadGroup, n_bh - grp * kHeadGroup);    // the last group may be smaller
         const int item = in_grp / g_heads;
         const int bh = grp * kHeadGroup + (in_grp - item * g_heads);
@@ -233,8 +255,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         hq = bh - b * prm.Hq;
         seq = b;
     } else {
-        const int grp = blockIdx.x / (kHeadGroup * prm.total_pairs);
-        const int in_grp = blockIdx.x - grp * (kHeadGroup * prm.total_pairs);
+        const int grp = blk / (kHeadGroup * prm.total_pairs);
+        const int in_grp = blk - grp * (kHeadGroup * prm.total_pairs);
         const int g_heads = min(kHeadGroup, prm.Hq - grp * kHeadGroup);
         const int item = in_grp / g_heads;                  // items are sorted by length on the host
         hq = grp * kHeadGroup + (in_grp - item * g_heads);
@@ -250,13 +272,18 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     }
     constexpr bool varlen = VL;
     const int hk = hq / (prm.Hq / prm.Hk);
-    // m: query-tile rows of this CTA (inside the sequence / the chunk); k: the key tile on their diagonal
-    // (m + the chunk's offset in the context)
+    // m: query tiles of this CTA (inside the sequence / the chunk).  A key tile is taken in steps of TH = 64 keys:
+    // d: the step on the diagonal of the tile's first row, u: the number of steps (D = 64: the tile's last 64 rows may
+    // not exist, and a chunk may begin in the middle of a key tile, so that number may be odd).
     const int kv_off = VL ? 0 : prm.kv_off;
-    const int mA = 2 * pr, mB = 2 * pr + 1;
-    const bool hasB = mB < n_rows;
-    const int kA = mA + kv_off, kB = mB + kv_off;
-    const int nkv = (hasB ? kB : kA) + 1;
+    const int n_tiles = SUB ? (n_rows + 1) >> 1 : n_rows;
+    const int mA = prm.solo ? 2 * pr + 1 - static_cast<int>(blockIdx.x & 1) : 2 * pr, mB = mA + 1;
+    if (prm.solo && mA >= n_tiles) return;
+    const bool hasB = !prm.solo && mB < n_tiles;
+    const int dA = SUB ? kv_off + 2 * mA : 2 * (mA + kv_off), dB = dA + 2;
+    const int uA = SUB ? kv_off + min(2 * mA + 2, n_rows) : dA + 2;
+    const int uB = SUB ? kv_off + min(2 * mB + 2, n_rows) : dB + 2;
+    const int nkv = ((hasB ? uB : uA) + 1) >> 1;
 
     // ---- shared memory ------------------------------------------------------------------
     const uint32_t bar0 = sbase + C::kOffBars;
@@ -335,38 +362,62 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             s_skip = skip_word;
         }
     }
-    // Schedule table, one 4-bit entry per key tile j (Sec. 4.2 lookup done once per CTA):
+    // Schedule table (Sec. 4.2 lookup done once per CTA).  D = 128, one 4-bit entry per key tile j:
     //   bit0 / bit1: tile A / tile B takes the INT8 route at key tile j  (R = (b >> floor(j/G)) & 1)
     //   bit2 / bit3: the FP16 / the INT8 copy of K_j has to be staged
-    // A thread makes eight consecutive entries.  Their groups lie in at most two mask words per row: the four words
-    // are loaded up front, so that the thread waits for one round trip, not for one per entry.
-    for (int i = static_cast<int>(threadIdx.x) - 32; i >= 0 && i * 8 < nkv; i += static_cast<int>(blockDim.x) - 32) {
-        const int j0 = i * 8, j_last = min(j0 + 7, nkv - 1);
+    // D = 64, one 4-bit entry per routing key tile: bit 2t + r is the route of row half r of tile t; entries of pairs
+    // above the diagonal or of rows that do not exist repeat a neighbour's, so that they ask for nothing.
+    // A thread makes eight consecutive entries.  Their groups lie in at most two mask words per row: the words of all
+    // rows are loaded up front, so that the thread waits for one round trip, not for one per entry.
+    const int n_entries = SUB ? 2 * nkv : nkv;
+    for (int i = static_cast<int>(threadIdx.x) - 32; i >= 0 && i * 8 < n_entries; i += static_cast<int>(blockDim.x) - 32) {
+        const int j0 = i * 8, j_last = min(j0 + 7, n_entries - 1);
+        constexpr int NR = SUB ? 4 : 2;                // routing rows of this CTA: mrow .. mrow + NR - 1
+        const int mrow = SUB ? 2 * mA : mA;
+        const int n_live = min(hasB ? NR : NR / 2, n_rows - mrow);
         int g = 0, in_g = 0, w_lo = 0;
-        uint32_t wa[2] = {0u, 0u}, wb[2] = {0u, 0u};
+        uint32_t wr[NR][2];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) wr[r][0] = wr[r][1] = 0u;
         if (prm.words != nullptr) {
             g = j0 / prm.G;
             in_g = j0 - g * prm.G;
             w_lo = g >> 5;
-            const int w_hi = (j_last / prm.G) >> 5;
+            const int w_hi = min((j_last / prm.G) >> 5, prm.W - 1);
             const int nbi = (prm.nb == 1) ? 0 : b;
-            const uint32_t* rowA = prm.words + ((static_cast<int64_t>(nbi) * prm.Hk + hk) * prm.mask_T_m + row0 + mA) * prm.W;
-            wa[0] = rowA[w_lo];
-            wa[1] = rowA[w_hi];
-            if (hasB) { wb[0] = rowA[prm.W + w_lo]; wb[1] = rowA[prm.W + w_hi]; }
+            const uint32_t* rowA = prm.words + ((static_cast<int64_t>(nbi) * prm.Hk + hk) * prm.mask_T_m + row0 + mrow) * prm.W;
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                if (r < n_live) { wr[r][0] = rowA[r * prm.W + w_lo]; wr[r][1] = rowA[r * prm.W + w_hi]; }
         }
-        uint32_t packed = 0u;
+        uint32_t packed = 0u, before = 0u;
         for (int jj = 0; jj < 8; ++jj) {
             const int j = j0 + jj;
             if (j > j_last) break;
             const bool hi = (g >> 5) != w_lo;              // (no mask words: all bits 0)
-            uint32_t e = ((hi ? wa[1] : wa[0]) >> (g & 31)) & 1u;
-            if (hasB) e |= (((hi ? wb[1] : wb[0]) >> (g & 31)) & 1u) << 1;
+            uint32_t e = 0u;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) e |= (((hi ? wr[r][1] : wr[r][0]) >> (g & 31)) & 1u) << r;
             if (++in_g == prm.G) { in_g = 0; ++g; }
-            const bool useA = j <= kA;
-            if ((useA && !(e & 1u)) || (hasB && !(e & 2u))) e |= 4u;
-            if ((useA && (e & 1u)) || (hasB && (e & 2u))) e |= 8u;
-            if (OTF && (e & 8u)) e |= 4u;   // the INT8 copy is made from the FP16 tile
+            if constexpr (SUB) {
+                // row r is live while j <= kv_off + mrow + r: the live rows are r_lo .. n_live - 1
+                const int r_lo = max(0, j - kv_off - mrow);
+                if (r_lo >= n_live) e = before;
+                else {
+                    const uint32_t first = (e >> r_lo) & 1u, last = (e >> (n_live - 1)) & 1u;
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        if (r < r_lo) e = (e & ~(1u << r)) | (first << r);
+                        else if (r >= n_live) e = (e & ~(1u << r)) | (last << r);
+                    }
+                }
+                before = e;
+            } else {
+                const bool useA = j <= mA + kv_off;
+                if ((useA && !(e & 1u)) || (hasB && !(e & 2u))) e |= 4u;
+                if ((useA && (e & 1u)) || (hasB && (e & 2u))) e |= 8u;
+                if (OTF && (e & 8u)) e |= 4u;   // the INT8 copy is made from the FP16 tile
+            }
             packed |= e << (4 * jj);
         }
         sched_s[i] = packed;
@@ -387,7 +438,16 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         if (warp == kMmaWarp) ptx::tmem_dealloc(tmem_base, C::kTmemCols);
         return;
     }
-    auto sched = [&](int j) -> uint32_t { return (sched_s[j >> 3] >> ((j & 7) * 4)) & 15u; };
+    // Entry of key tile j.  D = 64: bits 0-7 the two routing tiles' entries, bits 8 / 9 the copies to stage.
+    constexpr uint32_t kNeed16 = SUB ? 256u : 4u, kNeed8 = SUB ? 512u : 8u;
+    auto sched = [&](int j) -> uint32_t {
+        if constexpr (SUB) {
+            const uint32_t e = (sched_s[j >> 2] >> ((j & 3) * 8)) & 255u;
+            return e | (e != 255u ? kNeed16 : 0u) | (e != 0u ? kNeed8 : 0u);
+        } else {
+            return (sched_s[j >> 3] >> ((j & 7) * 4)) & 15u;
+        }
+    };
 
     if (OTF && warp >= kQuantWarp0) {
         // ================================================================ on-chip quantiser (on-the-fly mode)
@@ -478,8 +538,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             const uint32_t e = sched(n);
             uint32_t s16 = 0, s8 = 0;
             if (n >= 1) ring.take(C::kHalves);
-            if (e & 4u) s16 = ring.take(C::kHalves);
-            if (e & 8u) s8 = ring.take(1);
+            if (e & kNeed16) s16 = ring.take(C::kHalves);
+            if (e & kNeed8) s8 = ring.take(1);
             for (int t = 0; t < 2; ++t) {
                 if (!((e >> t) & 1u) || ((q8_made >> t) & 1u)) continue;
                 if (ok) ok = wait_bar(cx, bar_q(t), 0, kRoleQuant, t, kBarQ);
@@ -491,7 +551,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             }
             if (ok) ok = wait_bar(cx, bar_raw(n % kBundles), (n / kBundles) & 1, kRoleQuant, n, kBarRaw);
             ok = __all_sync(0xffffffffu, ok);
-            if (e & 8u) {
+            if (e & kNeed8) {
                 const float dk = quantise_tile(C::kOffRing + s16 * C::kChunk, C::kOffRing + s8 * C::kChunk);
                 if (cw == 0 && lane == 0) otf_dk[n % (2 * kBundles)] = dk;
             }
@@ -533,11 +593,11 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 uint32_t s16 = 0, s8 = 0, sv = 0, bytes = 0, raw_bytes = 0;
                 // On-the-fly mode: the FP16 K tile of a bundle with an INT8 tile to make is announced to the
                 // quantiser (bar_raw), not to the issuers; the INT8 chunk is only claimed, not filled.
-                const bool make8 = OTF && (e & 8u);
+                const bool make8 = OTF && (e & kNeed8);
                 // chunk order inside the sequence: ..., V_{n-1}, K16_n, K8_n, V_n, ...
                 if (has_v) { sv = ring.take(C::kHalves); bytes += C::kHalves * C::kChunk; }
-                if (e & 4u) { s16 = ring.take(C::kHalves); (make8 ? raw_bytes : bytes) += C::kHalves * C::kChunk; }
-                if (e & 8u) { s8 = ring.take(1); if (!OTF) bytes += C::kK8Bytes; }
+                if (e & kNeed16) { s16 = ring.take(C::kHalves); (make8 ? raw_bytes : bytes) += C::kHalves * C::kChunk; }
+                if (e & kNeed8) { s8 = ring.take(1); if (!OTF) bytes += C::kK8Bytes; }
                 if (bytes == 0u && raw_bytes == 0u) break;             // nothing after the last V
                 if (n == prm.test_drop_bundle) {   // testing aid: this bundle never lands, an issuer's bounded wait runs out
                     dropped = n;
@@ -570,14 +630,14 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     for (int c = 0; c < C::kHalves; ++c)
                         ptx::tma_load_4d(sbase + C::kOffRing + (sv + c) * C::kChunk, &tm_v16, bar, c * 64, tok0 + (n - 1) * T, hk, b);
                 }
-                if (e & 4u) {
+                if (e & kNeed16) {
                     claim(s16, C::kHalves);
                     if (!ok) break;
                     const uint32_t bar16 = make8 ? bar_raw(n % kBundles) : bar;
                     for (int c = 0; c < C::kHalves; ++c)
                         ptx::tma_load_4d(sbase + C::kOffRing + (s16 + c) * C::kChunk, &tm_k16, bar16, c * 64, tok0 + n * T, hk, b);
                 }
-                if (e & 8u) {
+                if (e & kNeed8) {
                     claim(s8, 1);
                     if (!ok) break;
                     if (!OTF) ptx::tma_load_4d(sbase + C::kOffRing + s8 * C::kChunk, &tm_k8, bar, 0, tok0 + n * T, hk, b);
@@ -606,7 +666,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         ptx::setmaxnreg_dec<OTF ? kRegsOtherOtf : kRegsOther>();
         {
             const int t = warp - kMmaWarp;
-            const int m_t = t ? kB : kA;       // last key tile of this issuer's query tile
+            const int u_t = t ? uB : uA;       // steps (key-tile halves) of this issuer's query tile
             constexpr int TH = C::kTH;
             constexpr uint32_t kIdescQK16 = ptx::instr_desc(1, 0, 0, 0, C::kM, TH);
             constexpr uint32_t kIdescQK8 = ptx::instr_desc(2, 1, 0, 0, C::kM, TH);
@@ -633,7 +693,33 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             // the rows of the K-major operand from byte h*TH*(row pitch) on (a whole number of swizzle atoms).
             auto issue_qk = [&](int t, int h, uint32_t int8_route, uint32_t s16, uint32_t s8) {
                 const uint32_t d_tmem = tmem_base + t * C::kSCols + h * TH;
-                if (int8_route) {
+                if constexpr (SUB) {
+                    // the two row halves' routes (bits 0 and 1): where they differ both products are issued, each
+                    // with the other half's accumulator lanes switched off
+                    const uint32_t a8 = ptx::desc_lo(sbase + C::kOffQ8 + t * C::kQ8Tile, 16);
+                    const uint32_t b8 = ring_lo + s8 * kChunkLo + ((h * TH * C::kI8RowBytes) >> 4);
+                    const uint32_t a16 = ptx::desc_lo(sbase + C::kOffQ16 + t * C::kQ16Tile, 16);
+                    const uint32_t b16 = ring_lo + s16 * kChunkLo + ((h * TH * 128) >> 4);
+                    static_assert(!SUB || C::kHalves == 1, "one 64-element slab");
+                    if (int8_route == 0u || int8_route == 3u) {
+                        if (int8_route) {
+                            ptx::mma_i8_ss<false>(d_tmem, a8, kHi8, b8, kHi8, kIdescQK8);
+                            ptx::mma_i8_ss<true>(d_tmem, a8 + 2, kHi8, b8 + 2, kHi8, kIdescQK8);
+                        } else {
+                            ptx::mma_f16_ss<false>(d_tmem, a16, kHi16, b16, kHi16, kIdescQK16);
+#pragma unroll
+                            for (int k = 1; k < 4; ++k) ptx::mma_f16_ss<true>(d_tmem, a16 + 2 * k, kHi16, b16 + 2 * k, kHi16, kIdescQK16);
+                        }
+                    } else {
+                        const uint32_t off_lo = int8_route == 1u ? 0xffffffffu : 0u;   // lanes 0-63 without FP16 scores
+                        ptx::mma_i8_ss_lanes<false>(d_tmem, a8, kHi8, b8, kHi8, kIdescQK8, ~off_lo, off_lo);
+                        ptx::mma_i8_ss_lanes<true>(d_tmem, a8 + 2, kHi8, b8 + 2, kHi8, kIdescQK8, ~off_lo, off_lo);
+                        ptx::mma_f16_ss_lanes<false>(d_tmem, a16, kHi16, b16, kHi16, kIdescQK16, off_lo, ~off_lo);
+#pragma unroll
+                        for (int k = 1; k < 4; ++k)
+                            ptx::mma_f16_ss_lanes<true>(d_tmem, a16 + 2 * k, kHi16, b16 + 2 * k, kHi16, kIdescQK16, off_lo, ~off_lo);
+                    }
+                } else if (int8_route) {
                     if constexpr (OTF) {
                         if (!q8_there) {
                             if (!wait_bar(cx, bar_q8(t), 0, kRoleMma, t, kBarQ8)) { ok = false; return; }
@@ -677,26 +763,26 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
 
             // slots of the K operands of the tile whose QK^T is issued next
             uint32_t e_next = sched(0), k16 = 0, k8 = 0;
-            uint32_t r_next = (e_next >> t) & 1u;          // route of this tile at the next key tile
-            if (e_next & 4u) k16 = ring.take(C::kHalves);
-            if (e_next & 8u) k8 = ring.take(1);
+            // route of this tile at half h of the key tile of entry e (D = 64: bits 0 / 1 = the two row halves)
+            auto route = [&](uint32_t e, int h) -> uint32_t { return SUB ? (e >> (4 * h + 2 * t)) & 3u : (e >> t) & 1u; };
+            if (e_next & kNeed16) k16 = ring.take(C::kHalves);
+            if (e_next & kNeed8) k8 = ring.take(1);
             acquire(0);
             if (ok) {
                 ptx::tc_fence_after_sync();
                 for (int h = 0; h < 2; ++h) {
-                    issue_qk(t, h, r_next, k16, k8);
+                    if (SUB && h >= u_t) break;
+                    issue_qk(t, h, route(e_next, h), k16, k8);
                     ptx::mma_commit(bar_s(t, h));
                 }
                 ptx::mma_commit(bar_empty(0));
             }
             for (int j = 0; j < nkv && ok; ++j) {
-                const bool mine = j <= m_t;            // tile A has no work at the last key tile of tile B
-                const bool more = j + 1 <= m_t;
+                const bool mine = 2 * j < u_t;         // tile A has no work at the last key tile of tile B
                 const uint32_t sv = ring.take(C::kHalves);
                 e_next = (j + 1 < nkv) ? sched(j + 1) : 0u;
-                r_next = (e_next >> t) & 1u;
-                if (e_next & 4u) k16 = ring.take(C::kHalves);
-                if (e_next & 8u) k8 = ring.take(1);
+                if (e_next & kNeed16) k16 = ring.take(C::kHalves);
+                if (e_next & kNeed8) k8 = ring.take(1);
                 // operands of this iteration (bundle j + 1): wait for them now, off the P -> PV critical path
                 acquire(j + 1);
                 if (!ok) break;
@@ -706,13 +792,14 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 if (mine) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
+                        if (SUB && 2 * j + h >= u_t) break;
                         if (!wait_bar(cx, bar_p(t, h), j & 1, kRoleMma, j, kBarP)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
                         issue_pv(t, h, sv, (j > 0 || h > 0) ? 1u : 0u);
-                        if (j == m_t && h == 0) ptx::mma_commit(bar_pv(t));   // the last-but-one PV (a rescale in the last step waits for it)
-                        if (j == m_t && h == 1) ptx::mma_commit(bar_o(t));
-                        if (more) {
-                            issue_qk(t, h, r_next, k16, k8);
+                        if (2 * j + h == u_t - 2) ptx::mma_commit(bar_pv(t));   // the last-but-one PV (a rescale in the last step waits for it)
+                        if (2 * j + h == u_t - 1) ptx::mma_commit(bar_o(t));
+                        if (2 * (j + 1) + h < u_t) {
+                            issue_qk(t, h, route(e_next, h), k16, k8);
                             ptx::mma_commit(bar_s(t, h));
                         }
                     }
@@ -728,11 +815,14 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         // ================================================================ softmax warps
         ptx::setmaxnreg_inc<OTF ? kRegsSoftmaxOtf : kRegsSoftmax>();
         const int quarter = warp & 3, t = (warp >> 2) & 1, sub = warp >> 3;
-        const int m_t = t ? mB : mA;           // query-tile row
-        const int k_t = t ? kB : kA;           // its diagonal key tile
+        const int m_t = t ? mB : mA;           // query tile
+        const int rh = SUB ? quarter >> 1 : 0;                                    // row half of this warp's rows
+        const int r_t = SUB ? min(2 * m_t + rh, n_rows - 1) : m_t;                // their routing row (clamped: rows that do not exist)
+        const int d_t = t ? dB : dA;           // step on the diagonal of the tile's first row
         if (t == 0 || hasB) {
             constexpr int TH = C::kTH;         // key columns per half step
             constexpr int NB = TH / 8;         // blocks of 8 columns per half step
+            static_assert(NB == 8, "shapes of the tensor-memory loads and stores below");
             // This thread holds two columns (cq, cq + 1 of every block of 8) of the rows rw[0] and rw[1] = rw[0] + 8
             // of the tile; the four lanes of a quad share a row.
             const int cq = 2 * (lane & 3);
@@ -746,8 +836,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             const float* dk_row = nullptr;
             if constexpr (!OTF) {
                 if (prm.has_int8) {
-                    dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + m_t) * prm.Hq + hq]
-                                : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.T_m + m_t];
+                    dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + r_t) * prm.Hq + hq]
+                                : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.T_m + r_t];
                     dk_row = varlen ? prm.k_scale + static_cast<int64_t>(kblk0) * prm.Hk + hk
                                     : prm.k_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.ks_blocks;
                 }
@@ -761,26 +851,39 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             // delta_K of the quantisation block a step's keys lie in (App. C "Quantization Granularity": a block is a
             // key tile or, with the paper's BLK_K = BLOCK_N / 2, one half of it -- exactly one step); the next block's
             // scale is read ahead of its use.  A block beyond the end of a ragged sequence holds no legal key.
+            // D = 64: a step is a routing key tile, with one scale or (KH) with one for each 32 keys.
             const bool k_half = prm.k_half_blocks != 0;
             auto load_dk = [&](int blk) { return (prm.has_int8 && !OTF && blk < n_kblk) ? dk_row[blk * dk_step] : 0.f; };
             float dk_cur = 0.f, dk_next = load_dk(0);
+            float dk_next_hi = KH ? load_dk(1) : 0.f, a_hi = prm.scale_log2;   // KH: of the step's keys 32 .. 63
             // VS: delta_V of the key tile (block = key tile) of the INT8 value cache the FP16 V operand was made from
             const float* dv_row = nullptr;
             if constexpr (VS) dv_row = prm.v_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.vs_blocks;
             float dv = 1.f;
             float a = prm.scale_log2;
             uint32_t int8_route = 0u;
-            const int n_steps = 2 * (k_t + 1);
+            const int n_steps = t ? uB : uA;
             // One step = one half (TH key columns) of a score tile: while the warps of this tile work on one half of
             // S_t, the tensor pipe runs the PV of the previous half and the QK^T of the next one into the other
             // half.  u = 2*j + h.
             for (int u = 0; u < n_steps; ++u) {
                 const int j = u >> 1, h = u & 1;
-                if (h == 0) int8_route = (sched(j) >> t) & 1u;
-                if constexpr (VS) { if (h == 0) dv = dv_row[j]; }
-                if (h == 0 || k_half) {
+                if constexpr (SUB) int8_route = (sched_s[u >> 3] >> ((u & 7) * 4 + 2 * t + rh)) & 1u;
+                else if (h == 0) int8_route = (sched(j) >> t) & 1u;
+                if constexpr (VS) { if (SUB || h == 0) dv = dv_row[SUB ? u : j]; }
+                if constexpr (KH) {
+                    a = a_hi = prm.scale_log2;
+                    if (int8_route) {
+                        a *= dq * dk_next;
+                        if (a == 0.f) a = 1.f;
+                        a_hi *= dq * dk_next_hi;
+                        if (a_hi == 0.f) a_hi = 1.f;
+                    }
+                    dk_next = load_dk(2 * u + 2);
+                    dk_next_hi = load_dk(2 * u + 3);
+                } else if (SUB || h == 0 || k_half) {
                     dk_cur = dk_next;
-                    dk_next = load_dk(k_half ? u + 1 : j + 1);
+                    dk_next = load_dk(SUB || k_half ? u + 1 : j + 1);
                     a = prm.scale_log2;
                     if (int8_route) {
                         a *= dq * dk_cur;
@@ -793,8 +896,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 uint32_t s[4 * NB];
-                if constexpr (NB == 8) ptx::tmem_ld16x256_x8(t_sh, s);
-                else ptx::tmem_ld16x256_x4(t_sh, s);
+                ptx::tmem_ld16x256_x8(t_sh, s);
                 if constexpr (OTF) {
                     // the key tile's scale was written by the quantiser before the issuer could start the
                     // MMAs whose result has just been seen
@@ -812,7 +914,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 }
 
                 // P = 2^(a*raw - m) is rounded to FP16, one pair per register.
-                const bool diag = (j == k_t);
+                const bool diag = u >= d_t + rh;
                 bool redo = diag || u == 0 || DBG;
                 bool stored = false;      // P of the one-pass form has been sent to tensor memory
                 float alpha[2] = {1.f, 1.f}, sum[2] = {0.f, 0.f};
@@ -823,6 +925,15 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     if (!int8_route) {
                         const float addend[2] = {-m_run[0], -m_run[1]};
                         softmax_step_fast<NB, kFp32, VS>(s, a, addend, p, sum, dv);
+                    } else if constexpr (KH) {
+                        if (fmaxf(a, a_hi) * kInt8Bias <= kFoldLimit) {
+                            const float addend[2] = {-__fmaf_rn(a, kInt8Bias, m_run[0]), -__fmaf_rn(a, kInt8Bias, m_run[1])};
+                            const float addend_hi[2] = {-__fmaf_rn(a_hi, kInt8Bias, m_run[0]), -__fmaf_rn(a_hi, kInt8Bias, m_run[1])};
+                            softmax_step_fast2<NB, kInt8Folded, VS>(s, a, addend, a_hi, addend_hi, p, sum, dv);
+                        } else {
+                            const float addend[2] = {-m_run[0], -m_run[1]};
+                            softmax_step_fast2<NB, kInt8Exact, VS>(s, a, addend, a_hi, addend, p, sum, dv);
+                        }
                     } else if (a * kInt8Bias <= kFoldLimit) {
                         // one explicit FMA: every instantiation of the kernel rounds the addend the same way
                         const float addend[2] = {-__fmaf_rn(a, kInt8Bias, m_run[0]), -__fmaf_rn(a, kInt8Bias, m_run[1])};
@@ -833,8 +944,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     }
                     // The store of P goes out before the vote, so that the vote's latency hides behind it; a rejected
                     // step stores again below, after this store has been waited for.
-                    if constexpr (NB == 8) ptx::tmem_st16x128_x8(t_sh, p);
-                    else ptx::tmem_st16x128_x4(t_sh, p);
+                    ptx::tmem_st16x128_x8(t_sh, p);
                     stored = true;
                     redo = __any_sync(0xffffffffu, !(sum[0] <= exp2f(kAccept) && sum[1] <= exp2f(kAccept)));   // also true for a NaN
                 }
@@ -846,34 +956,43 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         if (lane == 0) {
                             for (int e = 0; e < prm.dbg_n; ++e) {
                                 const int32_t* qd = prm.dbg_tiles + 4 * e;
-                                if (qd[0] == seq && qd[1] == hq && qd[2] == m_t && qd[3] == j) { idx = e; break; }
+                                if (qd[0] == seq && qd[1] == hq && qd[2] == (SUB ? 2 * m_t + rh : m_t) && qd[3] == (SUB ? u : j)) { idx = e; break; }
                             }
                         }
                         idx = __shfl_sync(0xffffffffu, idx, 0);
+                        if (SUB && (u > d_t + rh || 2 * m_t + rh >= n_rows)) idx = -1;   // above the diagonal / no such rows
                         if (idx >= 0) {
+                            constexpr int RT = C::kRT;
 #pragma unroll
                             for (int k = 0; k < 2; ++k) {
-                                if (rw[k] >= T) continue;
-                                int32_t* dst = prm.dbg_raw + (static_cast<int64_t>(idx) * T + rw[k]) * T + h * TH + cq;
+                                int32_t* dst = prm.dbg_raw + (static_cast<int64_t>(idx) * RT + (rw[k] & (RT - 1))) * RT + (SUB ? 0 : h * TH) + cq;
 #pragma unroll
                                 for (int i = 0; i < NB; ++i)
                                     *reinterpret_cast<uint2*>(dst + 8 * i) = make_uint2(s[4 * i + 2 * k], s[4 * i + 2 * k + 1]);
                             }
-                            if (rw[0] == 0 && cq == 0) prm.dbg_kind[idx] = static_cast<uint8_t>(int8_route);
+                            if ((rw[0] & (RT - 1)) == 0 && cq == 0) prm.dbg_kind[idx] = static_cast<uint8_t>(int8_route);
                         }
                     }
                     // Common FP32 score domain (App. C), causal legality on the diagonal tile (App. B:
                     // enforced kernel-side, independent of R), row maximum, then the exponentials.
                     float mx[2] = {-INFINITY, -INFINITY};
+                    float mx_lo[2] = {-INFINITY, -INFINITY};        // KH: of the step's keys 0 .. 31, scaled
+                    const int col0 = (u - d_t) * TH + cq;           // this thread's first column relative to the tile's first row
 #pragma unroll
                     for (int i = 0; i < NB; ++i) {
+                        if constexpr (KH) {
+                            if (i == NB / 2) {
+#pragma unroll
+                                for (int k = 0; k < 2; ++k) { mx_lo[k] = mx[k] * a; mx[k] = -INFINITY; }
+                            }
+                        }
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 const int c = 4 * i + 2 * k + e;
                                 float v = int8_route ? __int2float_rn(static_cast<int>(s[c])) : __uint_as_float(s[c]);
-                                if (diag && h * TH + 8 * i + cq + e > rw[k]) v = -INFINITY;
+                                if (diag && col0 + 8 * i + e > rw[k]) v = -INFINITY;
                                 s[c] = __float_as_uint(v);
                                 mx[k] = fmaxf(mx[k], v);
                             }
@@ -881,7 +1000,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     }
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
-                        const float m_step = quad_max(mx[k] * a);     // a >= 0, so max(a*raw) = a*max(raw)
+                        // a > 0, so max(a*raw) = a*max(raw)
+                        const float m_step = quad_max(KH ? fmaxf(mx_lo[k], mx[k] * a_hi) : mx[k] * a);
                         if (m_step > m_run[k] + kMove) {
                             alpha[k] = fast_exp2(m_run[k] - (m_step + kMargin));
                             m_run[k] = m_step + kMargin;
@@ -896,7 +1016,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {
                             const float2 t2 = __ffma2_rn(make_float2(__uint_as_float(s[4 * i + 2 * k]), __uint_as_float(s[4 * i + 2 * k + 1])),
-                                                         a2, make_float2(-m_run[k], -m_run[k]));
+                                                         KH && i >= NB / 2 ? make_float2(a_hi, a_hi) : a2, make_float2(-m_run[k], -m_run[k]));
                             const float2 pp = make_float2(fast_exp2(t2.x), fast_exp2(t2.y));
                             acc[k] = __fadd2_rn(acc[k], pp);
                             if constexpr (VS) p[2 * i + k] = pack_half2(pp.x * dv, pp.y * dv);
@@ -932,8 +1052,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 }
                 if (redo) {
                     if (stored) ptx::tmem_wait_st();      // (the rejected one-pass store, before the same columns are stored again)
-                    if constexpr (NB == 8) ptx::tmem_st16x128_x8(t_sh, p);
-                    else ptx::tmem_st16x128_x4(t_sh, p);
+                    ptx::tmem_st16x128_x8(t_sh, p);
                 }
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before_sync();
@@ -941,7 +1060,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             }
 
             if (ok) {
-                ok = wait_bar(cx, bar_o(t), 0, role, k_t + 1, kBarO);
+                ok = wait_bar(cx, bar_o(t), 0, role, (n_steps + 1) >> 1, kBarO);
                 ok = __all_sync(0xffffffffu, ok);
             }
             if (ok) {
@@ -952,7 +1071,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     const float z_row = quad_sum(z[k]);
                     const int i_loc = m_t * T + rw[k];                            // row inside the sequence
                     const int64_t i_glob = static_cast<int64_t>(tok0) + i_loc;    // row on the token axis
-                    const bool row_valid = rw[k] < T && i_loc < len;
+                    const bool row_valid = i_loc < len;
                     z[k] = row_valid ? 1.f / z_row : 0.f;
                     if (row_valid && cq == 0 && prm.lse != nullptr)
                         prm.lse[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.L + i_glob] = (m_run[k] + log2f(z_row)) * kLn2;
@@ -965,7 +1084,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     ptx::tmem_wait_ld_dep(o);
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
-                        if (z[k] == 0.f) continue;     // a row beyond the sequence (or the 64-row tile): not written
+                        if (z[k] == 0.f) continue;     // a row beyond the sequence: not written
                         __half* dst = dst0 + rw[k] * prm.os[2] + c * 32;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -1020,17 +1139,18 @@ int encode_map(EncodeTiledFn enc, CUtensorMap* tm, const void* base, int elem_by
     return static_cast<int>(r);
 }
 
-template <int D, int T>
+template <int D>
 int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, const int8_t* q8,
                 const int8_t* k8, const float* qs, const float* ks, const uint32_t* words, void* out,
                 float* lse, void* workspace, const tilemix_debug_t* dbg, cudaStream_t stream,
                 const VarlenDev* vl, int total_pairs, const float* v_scale) {
-    using C = Cfg<D, T>;
+    using C = Cfg<D>;
+    constexpr int T = C::T;
     EncodeTiledFn enc = nullptr;
     int rc = get_encoder(&enc);
     if (rc) return rc;
     const bool otf = (g.flags & TILEMIX_QUANT_ON_THE_FLY) != 0;
-    if (otf && (vl != nullptr || !(D == 128 && T == 128) || g.blk_k != g.tile_n)) return TILEMIX_ERR_UNSUPPORTED;
+    if (otf && (vl != nullptr || D != 128 || g.blk_k != g.tile_n)) return TILEMIX_ERR_UNSUPPORTED;
     if (v_scale != nullptr && (otf || vl != nullptr)) return TILEMIX_ERR_UNSUPPORTED;   // value-cache scales: dense, quantise-once
     const bool has8 = !(g.flags & TILEMIX_FORCE_FP16) && (q8 != nullptr || otf);
     CUtensorMap tq, tk, tv, tq8, tk8;
@@ -1082,20 +1202,30 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     cudaError_t e = cudaMemsetAsync(workspace, 0, kWorkspaceClearBytes, stream);
     if (e != cudaSuccess) return static_cast<int>(e);
     const bool dbg_on = prm.dbg_n > 0;
-    auto kernel = vl ? (dbg_on ? attention_kernel<D, T, true, false, false, true> : attention_kernel<D, T, true, false>)
-                     : (dbg_on ? attention_kernel<D, T, false, false, false, true> : attention_kernel<D, T, false, false>);
-    if constexpr (D == 128 && T == 128) {
-        if (otf) kernel = dbg_on ? attention_kernel<D, T, false, true, false, true> : attention_kernel<D, T, false, true>;
-    }
-    if (v_scale != nullptr) {
-        if (dbg_on) return TILEMIX_ERR_UNSUPPORTED;     // (the chunk against an INT8 value cache has no debug instance)
-        kernel = attention_kernel<D, T, false, false, true>;
+    if (v_scale != nullptr && dbg_on) return TILEMIX_ERR_UNSUPPORTED;     // (the chunk against an INT8 value cache has no debug instance)
+    auto pick = [&](auto kh) {
+        constexpr bool KH = decltype(kh)::value;
+        if (v_scale != nullptr) return attention_kernel<D, false, false, true, false, KH>;
+        return vl ? (dbg_on ? attention_kernel<D, true, false, false, true, KH> : attention_kernel<D, true, false, false, false, KH>)
+                  : (dbg_on ? attention_kernel<D, false, false, false, true, KH> : attention_kernel<D, false, false, false, false, KH>);
+    };
+    auto kernel = pick(std::false_type{});
+    if constexpr (D == 128) {
+        if (otf) kernel = dbg_on ? attention_kernel<D, false, true, false, true> : attention_kernel<D, false, true>;
+    } else {
+        if (prm.k_half_blocks) kernel = pick(std::true_type{});
     }
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
     if (e != cudaSuccess) return static_cast<int>(e);
-    const int64_t ctas = vl ? static_cast<int64_t>(g.Hq) * total_pairs
-                            : static_cast<int64_t>(g.B) * g.Hq * ((g.T_m + 1) / 2);
+    constexpr int kRowsPerCta = 2 * T / C::kRT;          // routing rows of a CTA
+    int64_t ctas = vl ? static_cast<int64_t>(g.Hq) * total_pairs
+                      : static_cast<int64_t>(g.B) * g.Hq * ceil_div(g.T_m, kRowsPerCta);
     if (ctas == 0) return TILEMIX_OK;   // only zero-length sequences
+    // A grid that leaves half of the SMs idle gives every tile a CTA (and special-function units) of its own: 8 heads x
+    // 1000 tokens, d = 128, whole step 42 -> 36 us; 4 x 2000 60 -> 50; 1 x 4096 87 -> 73; 4 x 1000, d = 64 40 -> 36.
+    // Beyond that line pairs win: they read every key tile once for two query tiles and still fit one wave.
+    prm.solo = 2 * ctas <= kSms ? 1 : 0;
+    if (prm.solo) ctas *= 2;
     if (ctas > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
     // The register split inside the kernel (setmaxnreg) assumes what the block is launched with; a build that
     // gave the kernel fewer registers must not run (an increase beyond the block's allotment never returns).
@@ -1115,10 +1245,10 @@ int launch_attention(const Geometry& g, const void* q, const void* k, const void
                      float* lse, void* workspace, const tilemix_debug_t* dbg, cudaStream_t stream,
                      const VarlenDev* vl, int total_pairs, const float* v_scale) {
     if (g.d == 128 && g.tile_m == 128)
-        return launch_impl<128, 128>(g, q, k, v, q8, k8, qs, ks, words, out, lse, workspace, dbg, stream, vl,
+        return launch_impl<128>(g, q, k, v, q8, k8, qs, ks, words, out, lse, workspace, dbg, stream, vl,
                                      total_pairs, v_scale);
     if (g.d == 64 && g.tile_m == 64)
-        return launch_impl<64, 64>(g, q, k, v, q8, k8, qs, ks, words, out, lse, workspace, dbg, stream, vl,
+        return launch_impl<64>(g, q, k, v, q8, k8, qs, ks, words, out, lse, workspace, dbg, stream, vl,
                                    total_pairs, v_scale);
     return TILEMIX_ERR_UNSUPPORTED;
 }

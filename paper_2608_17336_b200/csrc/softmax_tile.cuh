@@ -50,19 +50,14 @@ __device__ __forceinline__ float quad_sum(float v) {
 enum ScoreKind : int { kFp32 = 0, kInt8Exact = 1, kInt8Folded = 2 };
 constexpr float kInt8Bias = 12582912.f;   // 1.5 * 2^23
 
-// One interior step (NB blocks of 8 key columns, no causal mask) in one pass with the current running
-// maxima: raw accumulators s -> P = 2^(a*raw - m) rounded to FP16 (p[2i + k] = the pair of row k in block
-// i) and this thread's part of the FP32 row sums.  addend[k] = -m_k (kFp32, kInt8Exact) or -(m_k + a*1.5*2^23)
-// (kInt8Folded).  VS: the probabilities are multiplied by `dv` (the block scale of an INT8 value cache, App. C:
-// folded into the probability tile) before they are rounded to FP16; the row sums are of the unscaled values.
-template <int NB, int KIND, bool VS = false>
-__device__ __forceinline__ void softmax_step_fast(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2],
-                                                  uint32_t (&p)[2 * NB], float (&sum)[2], float dv = 1.f) {
+// Blocks I0 .. I1 - 1 of a step of NB, see softmax_step_fast; acc = packed partial row sums.
+template <int I0, int I1, int NB, int KIND, bool VS>
+__device__ __forceinline__ void softmax_blocks(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2],
+                                               uint32_t (&p)[2 * NB], float2 (&acc)[2], float dv) {
     const float2 a2 = make_float2(a, a);
     const float2 unbias = make_float2(-kInt8Bias, -kInt8Bias);
-    float2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
+    for (int i = I0; i < I1; ++i) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const uint32_t r0 = s[4 * i + 2 * k], r1 = s[4 * i + 2 * k + 1];
@@ -84,6 +79,30 @@ __device__ __forceinline__ void softmax_step_fast(const uint32_t (&s)[4 * NB], f
             }
         }
     }
+}
+
+// One interior step (NB blocks of 8 key columns, no causal mask) in one pass with the current running
+// maxima: raw accumulators s -> P = 2^(a*raw - m) rounded to FP16 (p[2i + k] = the pair of row k in block
+// i) and this thread's part of the FP32 row sums.  addend[k] = -m_k (kFp32, kInt8Exact) or -(m_k + a*1.5*2^23)
+// (kInt8Folded).  VS: the probabilities are multiplied by `dv` (the block scale of an INT8 value cache, App. C:
+// folded into the probability tile) before they are rounded to FP16; the row sums are of the unscaled values.
+template <int NB, int KIND, bool VS = false>
+__device__ __forceinline__ void softmax_step_fast(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2],
+                                                  uint32_t (&p)[2 * NB], float (&sum)[2], float dv = 1.f) {
+    float2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    softmax_blocks<0, NB, NB, KIND, VS>(s, a, addend, p, acc, dv);
+    sum[0] = acc[0].x + acc[0].y;
+    sum[1] = acc[1].x + acc[1].y;
+}
+
+// The same with one scaling factor (and addend) for the first and one for the second half of the columns.
+template <int NB, int KIND, bool VS = false>
+__device__ __forceinline__ void softmax_step_fast2(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2], float a_hi,
+                                                   const float (&addend_hi)[2], uint32_t (&p)[2 * NB], float (&sum)[2],
+                                                   float dv = 1.f) {
+    float2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    softmax_blocks<0, NB / 2, NB, KIND, VS>(s, a, addend, p, acc, dv);
+    softmax_blocks<NB / 2, NB, NB, KIND, VS>(s, a_hi, addend_hi, p, acc, dv);
     sum[0] = acc[0].x + acc[0].y;
     sum[1] = acc[1].x + acc[1].y;
 }

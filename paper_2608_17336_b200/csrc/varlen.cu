@@ -47,6 +47,7 @@ int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geome
     int32_t* blkq = tile + (n + 1);
     int32_t* blkk = blkq + (n + 1);
     std::vector<int32_t> pair(static_cast<size_t>(n) + 1u, 0);
+    const int rows_per_cta = g->tile_m == 64 ? 4 : 2;   // the attention kernel's work item: two tiles of 128 queries
     int64_t longest = 0;
     for (int s = 0; s < n; ++s) {
         const int64_t len = static_cast<int64_t>(cu[s + 1]) - cu[s];
@@ -55,7 +56,7 @@ int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geome
         const int64_t rows = ceil_div(len, g->tile_m);
         tok[s] = cu[s];
         tile[s + 1] = tile[s] + static_cast<int32_t>(rows);
-        pair[s + 1] = pair[s] + static_cast<int32_t>((rows + 1) / 2);
+        pair[s + 1] = pair[s] + static_cast<int32_t>(ceil_div(rows, rows_per_cta));
         blkq[s + 1] = blkq[s] + static_cast<int32_t>(ceil_div(len, g->blk_q));
         blkk[s + 1] = blkk[s] + static_cast<int32_t>(ceil_div(len, g->blk_k));
     }
@@ -68,7 +69,7 @@ int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geome
     t->total_blk_q = blkq[n];
     t->total_blk_k = blkk[n];
     // Work items of the attention kernel, the longest rows of the whole batch first (a pair p of a
-    // sequence streams 2p + 2 key tiles); ties keep the sequence order.
+    // sequence streams 2p + 2 tiles of 128 keys); ties keep the sequence order.
     std::vector<std::pair<int32_t, int32_t>> items;   // (pair index, sequence)
     items.reserve(static_cast<size_t>(t->total_pairs));
     for (int s = 0; s < n; ++s)
