@@ -38,6 +38,7 @@ namespace {
 constexpr int kSoftmaxWarps = 16;         // 8 per query tile, 16 rows each
 constexpr int kProducerWarp = 16;
 constexpr int kMmaWarp = 17;
+constexpr int kScaleWarp = 19;
 // setmaxnreg only moves registers inside what the block was launched with (threads x registers per thread); an
 // increase beyond that waits for ever.  640 threads start with 96 registers: 512*104 + 128*64 = 61440 = 640*96.
 constexpr int kThreads = 640;
@@ -110,7 +111,10 @@ struct Cfg {
     static constexpr int kTH = T / 2;                 // key columns per half step
     static constexpr int kNumBars = 2 + 2 * kRing + 4 + 4 + 2 + 2 + 1 + kBundles + 2;
     static constexpr int kOffMisc = kOffBars + kNumBars * 8;       // tmem base, abort flag; on-chip scales
-    static constexpr int kOffWords = kOffMisc + 64;
+    // ring of the softmax warps' scaling factors: kScSlots key tiles of kScStride floats (see the scale warp)
+    static constexpr int kScSlots = 16, kScStride = kSub ? 32 : 8;
+    static constexpr int kOffSc = kOffMisc + 64;
+    static constexpr int kOffWords = kOffSc + kScSlots * kScStride * 4;
     static constexpr int kSmemBytes = kOffWords + kMaxTiles / 2;   // 4-bit schedule entries
     static constexpr int kSmemAlloc = kSmemBytes + 1024;           // slack to align the base
     static_assert(kK8Bytes <= kChunk, "INT8 key tile must fit one ring chunk");
@@ -305,11 +309,14 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     auto bar_raw = [&](int i) { return bar0 + 8u * (15 + 2 * kRing + i); };
     auto bar_q8 = [&](int t) { return bar0 + 8u * (15 + 2 * kRing + kBundles + t); };
     uint32_t* misc = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);   // [0] tmem base, [1] abort
-    // on-the-fly mode: delta_K of bundle n at otf_dk[n % (2 kBundles)] (a slot is rewritten only after
-    // bundle n + kBundles has been consumed, i.e. long after both groups finished key tile n), delta_Q of
-    // query tile t at otf_dq[t]
-    volatile float* otf_dk = reinterpret_cast<volatile float*>(misc + 4);
-    volatile float* otf_dq = reinterpret_cast<volatile float*>(misc + 12);
+    // Scaling factors of the softmax steps.  Key tile j's are in slot j % kScSlots, written before bundle j's "landed"
+    // barrier completes; by then bundle j - 2 kBundles has been consumed, so every softmax warp is past key tile
+    // j - 2 kBundles - 1 and the slot is free.  Factor of (half h, tile t, row half r, 32-key half q): index
+    // h * 2 + t (D = 128) or ((h * 2 + t) * 2 + r) * (KH ? 2 : 1) + q; its sign bit set: INT8 route.  Then, with VS,
+    // delta_V of the two halves.
+    constexpr int kNumSc = SUB ? (KH ? 16 : 8) : 4;
+    static_assert(kNumSc + 2 <= C::kScStride && C::kScSlots > 2 * kBundles, "ring of scaling factors");
+    volatile float* sc_s = reinterpret_cast<volatile float*>(smem + C::kOffSc);
     uint32_t* sched_s = reinterpret_cast<uint32_t*>(smem + C::kOffWords);
     Ctx cx{reinterpret_cast<volatile int*>(&misc[1]), prm.status, prm.wait_limit_ns};
 
@@ -326,7 +333,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             // on-the-fly mode: one more arrival per quantiser warp on "landed" (after it made its rows of the bundle's
             // INT8 tile, if there is one to make); "raw": K16 bytes expected + "INT8 chunk claimed"
             const int i = (lane - 1) / 3, which = (lane - 1) % 3;
-            if (which == 0) ptx::mbar_init(bar_full(i), OTF ? 1 + kQuantWarps : 1);
+            if (which == 0) ptx::mbar_init(bar_full(i), OTF ? 1 + kQuantWarps : 2);   // (producer, scale warp)
             else if (which == 1) ptx::mbar_init(bar_empty(i), hasB ? 2 : 1);   // one arrival per MMA issuer
             else ptx::mbar_init(bar_raw(i), 2);
         } else if (lane <= 3 * kBundles + 2) {
@@ -449,6 +456,13 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         }
     };
 
+    // scaling factor of the raw scores on one route; a zero block's accumulators are all 0, any factor will do
+    auto factor = [&](uint32_t int8_route, float dq, float dk) -> float {
+        if (!int8_route) return prm.scale_log2;
+        const float a = prm.scale_log2 * (dq * dk);
+        return a == 0.f ? -1.f : -a;
+    };
+
     if (OTF && warp >= kQuantWarp0) {
         // ================================================================ on-chip quantiser (on-the-fly mode)
         // Four warps make the INT8 copies the tensor pipe reads: of a query tile before the first key tile it
@@ -534,6 +548,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         // ahead of it and the phase it waits for is unambiguous.
         Ring ring;   // the producer's sequence of chunks
         uint32_t q8_made = 0u;
+        volatile float* dq_s = reinterpret_cast<volatile float*>(misc + 12);   // delta_Q of the two query tiles
         for (int n = 0; n < nkv; ++n) {
             const uint32_t e = sched(n);
             uint32_t s16 = 0, s8 = 0;
@@ -545,17 +560,76 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 if (ok) ok = wait_bar(cx, bar_q(t), 0, kRoleQuant, t, kBarQ);
                 ok = __all_sync(0xffffffffu, ok);
                 const float dq = quantise_tile(C::kOffQ16 + t * C::kQ16Tile, C::kOffQ8 + t * C::kQ8Tile);
-                if (cw == 0 && lane == 0) otf_dq[t] = dq;
+                if (cw == 0 && lane == 0) dq_s[t] = dq;
                 publish(bar_q8(t));
                 q8_made |= 1u << t;
             }
             if (ok) ok = wait_bar(cx, bar_raw(n % kBundles), (n / kBundles) & 1, kRoleQuant, n, kBarRaw);
             ok = __all_sync(0xffffffffu, ok);
-            if (e & kNeed8) {
-                const float dk = quantise_tile(C::kOffRing + s16 * C::kChunk, C::kOffRing + s8 * C::kChunk);
-                if (cw == 0 && lane == 0) otf_dk[n % (2 * kBundles)] = dk;
-            }
+            float dk = 0.f;
+            if (e & kNeed8) dk = quantise_tile(C::kOffRing + s16 * C::kChunk, C::kOffRing + s8 * C::kChunk);
+            if (cw == 0 && lane < kNumSc)
+                sc_s[(n % C::kScSlots) * C::kScStride + lane] = factor((e >> (lane & 1)) & 1u, dq_s[lane & 1], dk);
             publish(bar_full(n % kBundles));
+        }
+    } else if (warp == kScaleWarp && !OTF) {
+        // ================================================================ scale warp
+        // Works out what the softmax warps multiply their accumulators with -- softmax scale, delta_Q and delta_K by
+        // route -- ahead of the MMAs, one lane per factor (and delta_V of an INT8 value cache), so that their loop
+        // has one shared-memory read in place of the route lookup, the scale loads and their arithmetic: in that
+        // loop every instruction costs about ten clocks of a ~1650 clk step.
+        // delta_K is that of the quantisation block the keys lie in (App. C "Quantization Granularity": a block is a
+        // routing key tile or, with the paper's BLK_K = BLOCK_N / 2, half of one).  A block beyond the end of a ragged
+        // sequence holds no legal key.
+        ptx::setmaxnreg_dec<kRegsOther>();
+        const int h = SUB ? lane / (KH ? 8 : 4) & 1 : lane >> 1 & 1, t = SUB ? lane / (KH ? 4 : 2) & 1 : lane & 1;
+        const int rh = SUB ? lane / (KH ? 2 : 1) & 1 : 0, q = KH ? lane & 1 : 0;
+        const int row = min(SUB ? 2 * (t ? mB : mA) + rh : (t ? mB : mA), n_rows - 1);   // (rows that do not exist: any)
+        const bool k_half = prm.k_half_blocks != 0;
+        const bool mine = lane < kNumSc && prm.has_int8;
+        // scales: dense [B,H,blocks] (unit stride over blocks), variable-length [blocks, H]
+        float dq = 0.f;
+        if (mine) dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + row) * prm.Hq + hq]
+                              : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.T_m + row];
+        const float* dk_row = varlen ? prm.k_scale + static_cast<int64_t>(kblk0) * prm.Hk + hk
+                                     : prm.k_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.ks_blocks;
+        const float* dv_row = VS ? prm.v_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.vs_blocks : nullptr;
+        auto load = [&](int n) -> float {
+            if (mine) {
+                const int blk = SUB ? (KH ? 4 * n + 2 * h + q : 2 * n + h) : (k_half ? 2 * n + h : n);
+                return n < nkv && blk < n_kblk ? dk_row[static_cast<int64_t>(blk) * (varlen ? prm.Hk : 1)] : 0.f;
+            }
+            if (VS && lane >= kNumSc && lane < kNumSc + 2) {
+                const int blk = SUB ? 2 * n + lane - kNumSc : n;
+                return n < nkv && blk < prm.vs_blocks ? dv_row[blk] : 0.f;
+            }
+            return 0.f;
+        };
+        float next = load(0);
+        for (int n = 0; n <= nkv; ++n) {
+            const float cur = next;
+            next = load(n + 1);
+            bool ok = true;
+            if (n >= kBundles) {
+                // Its barrier's last phase is over.  (The issuers' own waits record a copy that never lands, hence the
+                // longer limit.)  Bundle n has been started only if bundle n - kBundles landed, so this warp owes the
+                // "landed" barriers of a CTA that gives up nothing but what copies in flight still complete: it goes on
+                // for as long as they do, and never arrives ahead of a phase.
+                const Ctx late{cx.abort_flag, cx.status, 4 * cx.wait_limit_ns};
+                const uint32_t bar = bar_full(n % kBundles), parity = (n / kBundles - 1) & 1;
+                ok = wait_bar(late, bar, parity, kRoleProducer, n, kBarRingFull);
+                for (int it = 0; !ok && it < (1 << 12); ++it) ok = ptx::mbar_try_wait(bar, parity);
+                ok = __all_sync(0xffffffffu, ok);
+            }
+            if (!ok) break;
+            if (n < nkv) {
+                const uint32_t e = sched(n);
+                const uint32_t r = SUB ? (e >> (4 * h + 2 * t + rh)) & 1u : (e >> t) & 1u;
+                if (lane < kNumSc + (VS ? 2 : 0))
+                    sc_s[(n % C::kScSlots) * C::kScStride + lane] = lane < kNumSc ? factor(r, dq, cur) : cur;
+            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar_full(n % kBundles));
         }
     } else if (warp >= kMmaWarp + 2 || (warp == kMmaWarp + 1 && !hasB)) {
         ptx::setmaxnreg_dec<OTF ? kRegsOtherOtf : kRegsOther>();   // idle warps of the third warpgroup
@@ -830,89 +904,34 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(quarter * 32 + sub * 16) << 16);
             const uint32_t t_s = lane_base + t * C::kSCols;
             const uint32_t t_o = lane_base + 2 * C::kSCols + t * C::kOCols;
-            // scales: dense [B,H,T_m] (unit stride over blocks), variable-length [blocks, H]
-            const int64_t dk_step = varlen ? prm.Hk : 1;
-            float dq = 0.f;
-            const float* dk_row = nullptr;
-            if constexpr (!OTF) {
-                if (prm.has_int8) {
-                    dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + r_t) * prm.Hq + hq]
-                                : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.T_m + r_t];
-                    dk_row = varlen ? prm.k_scale + static_cast<int64_t>(kblk0) * prm.Hk + hk
-                                    : prm.k_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.ks_blocks;
-                }
-            }
             // Shared online-softmax state (Sec. 3.1), log2 domain, per row: running maximum m (identical in the four
             // lanes of the row's quad) and this lane's part of the normaliser z.
             float m_run[2] = {-INFINITY, -INFINITY}, z[2] = {0.f, 0.f};
             bool ok = true;
             const int role = t ? kRoleSoftmaxB : kRoleSoftmaxA;
-            bool dq_there = !OTF;   // on-the-fly mode: this tile's scale comes from the on-chip quantiser
-            // delta_K of the quantisation block a step's keys lie in (App. C "Quantization Granularity": a block is a
-            // key tile or, with the paper's BLK_K = BLOCK_N / 2, one half of it -- exactly one step); the next block's
-            // scale is read ahead of its use.  A block beyond the end of a ragged sequence holds no legal key.
-            // D = 64: a step is a routing key tile, with one scale or (KH) with one for each 32 keys.
-            const bool k_half = prm.k_half_blocks != 0;
-            auto load_dk = [&](int blk) { return (prm.has_int8 && !OTF && blk < n_kblk) ? dk_row[blk * dk_step] : 0.f; };
-            float dk_cur = 0.f, dk_next = load_dk(0);
-            float dk_next_hi = KH ? load_dk(1) : 0.f, a_hi = prm.scale_log2;   // KH: of the step's keys 32 .. 63
-            // VS: delta_V of the key tile (block = key tile) of the INT8 value cache the FP16 V operand was made from
-            const float* dv_row = nullptr;
-            if constexpr (VS) dv_row = prm.v_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.vs_blocks;
-            float dv = 1.f;
-            float a = prm.scale_log2;
-            uint32_t int8_route = 0u;
+            // this warp's scaling factors in the ring (see there)
+            const uint32_t sc0 = SUB ? (2 * t + rh) * (KH ? 2 : 1) : t;
             const int n_steps = t ? uB : uA;
             // One step = one half (TH key columns) of a score tile: while the warps of this tile work on one half of
             // S_t, the tensor pipe runs the PV of the previous half and the QK^T of the next one into the other
             // half.  u = 2*j + h.
             for (int u = 0; u < n_steps; ++u) {
                 const int j = u >> 1, h = u & 1;
-                if constexpr (SUB) int8_route = (sched_s[u >> 3] >> ((u & 7) * 4 + 2 * t + rh)) & 1u;
-                else if (h == 0) int8_route = (sched(j) >> t) & 1u;
-                if constexpr (VS) { if (SUB || h == 0) dv = dv_row[SUB ? u : j]; }
-                if constexpr (KH) {
-                    a = a_hi = prm.scale_log2;
-                    if (int8_route) {
-                        a *= dq * dk_next;
-                        if (a == 0.f) a = 1.f;
-                        a_hi *= dq * dk_next_hi;
-                        if (a_hi == 0.f) a_hi = 1.f;
-                    }
-                    dk_next = load_dk(2 * u + 2);
-                    dk_next_hi = load_dk(2 * u + 3);
-                } else if (SUB || h == 0 || k_half) {
-                    dk_cur = dk_next;
-                    dk_next = load_dk(SUB || k_half ? u + 1 : j + 1);
-                    a = prm.scale_log2;
-                    if (int8_route) {
-                        a *= dq * dk_cur;
-                        if (a == 0.f) a = 1.f;   // a zero block: every accumulator is 0 already
-                    }
-                }
                 const uint32_t t_sh = t_s + h * TH;
-                ok = wait_bar(cx, bar_s(t, h), j & 1, role, j, kBarS);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                if (!__all_sync(0xffffffffu, ptx::mbar_try_wait(bar_s(t, h), j & 1))) {
+                    ok = wait_bar(cx, bar_s(t, h), j & 1, role, j, kBarS);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
                 ptx::tc_fence_after_sync();
                 uint32_t s[4 * NB];
                 ptx::tmem_ld16x256_x8(t_sh, s);
-                if constexpr (OTF) {
-                    // the key tile's scale was written by the quantiser before the issuer could start the
-                    // MMAs whose result has just been seen
-                    if (h == 0 && int8_route) {
-                        if (!dq_there) {
-                            ok = wait_bar(cx, bar_q8(t), 0, role, m_t, kBarQ8);   // long over: S of an INT8 tile is there
-                            ok = __all_sync(0xffffffffu, ok);
-                            if (!ok) break;
-                            dq = otf_dq[t];
-                            dq_there = true;
-                        }
-                        a = prm.scale_log2 * (dq * otf_dk[j % (2 * kBundles)]);   // same rounding order as with scales from memory
-                        if (a == 0.f) a = 1.f;
-                    }
-                }
-
+                // the factors were written before the issuer could start the MMAs whose result has just been seen
+                const volatile float* sc = sc_s + (j % C::kScSlots) * C::kScStride + sc0 + h * (kNumSc / 2);
+                const float sc_a = sc[0];
+                const uint32_t int8_route = __float_as_uint(sc_a) >> 31;
+                const float a = fabsf(sc_a), a_hi = KH ? fabsf(sc[1]) : a;
+                const float dv = VS ? sc_s[(j % C::kScSlots) * C::kScStride + kNumSc + h] : 1.f;
                 // P = 2^(a*raw - m) is rounded to FP16, one pair per register.
                 const bool diag = u >= d_t + rh;
                 bool redo = diag || u == 0 || DBG;
