@@ -506,36 +506,35 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             amax = max(max(xch_slot(0), xch_slot(1)), max(xch_slot(2), xch_slot(3)));
             ptx::bar_sync_named(kQuantBar, kQuantWarps * 32);   // all have read: the slots may be written again
             const float amax_f = __half2float(__ushort_as_half(static_cast<unsigned short>(amax)));
-            const float delta = __fdiv_rn(amax_f, 127.0f);
-            if (!ok) return delta;
-            if (amax == 0u) {   // zero block: delta = 0, every code 0
-                for (int i = lane; i < kRowsW * D / 16; i += 32)
-                    *reinterpret_cast<uint4*>(dst + cw * kRowsW * 128 + i * 16) = make_uint4(0u, 0u, 0u, 0u);
-                return delta;
-            }
-            const float rdelta = __frcp_rn(delta);
+            QuantScale qs = quant_scale(amax_f);
+            if (!ok) return qs.delta;
+            if (amax == 0u) qs.r = 0.f, qs.refine = false;   // zero block: delta = 0, every code 0
+            auto convert = [&](auto refine) {
 #pragma unroll
-            for (int sl = 0; sl < C::kHalves; ++sl) {
+                for (int sl = 0; sl < C::kHalves; ++sl) {
 #pragma unroll
-                for (int u0 = 0; u0 < kVecW / 32; u0 += 4) {   // four vectors in flight per lane
-                    uint4 v[4];
+                    for (int u0 = 0; u0 < kVecW / 32; u0 += 4) {   // four vectors in flight per lane
+                        uint4 v[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        v[u] = *reinterpret_cast<const uint4*>(src + (sl * 1024 + cw * kVecW + lane + 32 * (u0 + u)) * 16);
-                    uint2 qv[4];
+                        for (int u = 0; u < 4; ++u)
+                            v[u] = *reinterpret_cast<const uint4*>(src + (sl * 1024 + cw * kVecW + lane + 32 * (u0 + u)) * 16);
+                        uint2 qv[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) qv[u] = quant8_div(v[u], delta, rdelta);
+                        for (int u = 0; u < 4; ++u) qv[u] = quant8<decltype(refine)::value>(v[u], qs);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = cw * kVecW + lane + 32 * (u0 + u);          // vector of the slab
-                        const int r = i >> 3, cl = (i & 7) ^ (r & 7);             // row, logical chunk of the slab
-                        // elements 64 sl + 8 cl .. + 7 of row r: byte column 64 sl + 8 cl of the INT8 row
-                        const int c16 = sl * 4 + (cl >> 1);
-                        *reinterpret_cast<uint2*>(dst + r * 128 + ((c16 ^ (r & 7)) << 4) + (cl & 1) * 8) = qv[u];
+                        for (int u = 0; u < 4; ++u) {
+                            const int i = cw * kVecW + lane + 32 * (u0 + u);          // vector of the slab
+                            const int r = i >> 3, cl = (i & 7) ^ (r & 7);             // row, logical chunk of the slab
+                            // elements 64 sl + 8 cl .. + 7 of row r: byte column 64 sl + 8 cl of the INT8 row
+                            const int c16 = sl * 4 + (cl >> 1);
+                            *reinterpret_cast<uint2*>(dst + r * 128 + ((c16 ^ (r & 7)) << 4) + (cl & 1) * 8) = qv[u];
+                        }
                     }
                 }
-            }
-            return delta;
+            };
+            if (qs.refine) convert(std::true_type{});
+            else convert(std::false_type{});
+            return qs.delta;
         };
         // hand-over to the async proxy (the tensor pipe reads shared memory through it), then one arrival per warp
         auto publish = [&](uint32_t bar) {

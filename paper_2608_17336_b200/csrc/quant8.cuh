@@ -14,35 +14,54 @@ __device__ __forceinline__ uint32_t habs2_bits(uint32_t v) { return v & 0x7fff7f
 // bit patterns order like unsigned integers.
 __device__ __forceinline__ uint32_t umax2(uint32_t a, uint32_t b) { return __vmaxu2(a, b); }
 
-// The definition: IEEE quotient x / delta, rounded to the nearest integer, ties to even.
-__device__ __forceinline__ int quant1_exact(float x, float delta) {
-    int q = __float2int_rn(__fdiv_rn(x, delta));
-    return max(-127, min(127, q));
+// Scale of a block and what its codes are made with.  The definition is RN_int(RN(x / delta)), delta = RN(amax / 127);
+// the codes are taken from ONE fused multiply-add, x * r + 1.5 * 2^23 (round-to-nearest-even puts the integer in the low
+// mantissa bits, so the low byte of the sum IS the two's-complement INT8 code), which rounds x * r to the nearest
+// integer exactly.  The two can only differ where the quotient is within ~2^-23 of a half-integer.  127 x / amax is a
+// ratio of 11-bit integers and a power of two, so apart from exact half-integers it keeps a relative distance of at
+// least 1 / (255 * 2048) from them.  Exact half-integers: 254 x = (2k + 1) amax, that is x = +-amax / 2 (k = 63), or 127
+// divides amax's mantissa.
+//  - x = amax / 2: the definition gives 64 if RN(x / delta) >= 63.5, else 63; r = RN(1 / delta) is moved by one unit in
+//    the last place where x * r falls on the other side of 63.5;
+//  - 127 divides the mantissa (then delta is exact; 8 of 1024 mantissas): `refine`, the quotient itself -- q0 = x * r,
+//    then q0 + (x - delta * q0) * r with the residual exact in one FMA -- before the rounding.
+// Both forms equal the definition for every binary16 amax and every |x| <= amax (all 5e8 pairs compared on the CPU).
+// amax = inf or NaN: r = 0 or NaN, `refine` stays off.
+struct QuantScale {
+    float delta, r;
+    bool refine;
+};
+__device__ __forceinline__ QuantScale quant_scale(float amax) {
+    QuantScale s;
+    s.delta = __fdiv_rn(amax, 127.0f);
+    s.r = __frcp_rn(s.delta);
+    const float half = 0.5f * amax;
+    // RN(half / delta) >= 63.5, from the exact residual: the quotient is at most half a unit (2^-19) below 63.5
+    const bool up = __fmaf_rn(-63.5f, s.delta, half) >= -1.9073486328125e-6f * s.delta;
+    const float side = __fmaf_rn(half, s.r, -63.5f);
+    if (up && side < 0.f) s.r = __uint_as_float(__float_as_uint(s.r) + 1u);
+    if (!up && side >= 0.f) s.r = __uint_as_float(__float_as_uint(s.r) - 1u);
+    s.refine = __fmaf_rn(127.f, s.delta, -amax) == 0.f || (__fmaf_rn(half, s.r, -63.5f) >= 0.f) != up;
+    return s;
 }
 
-// Same result without a division per element.  t = x * fl(1/delta) is within 2.3e-5 of the IEEE
-// quotient (|quotient| <= 127.5), so both round to the same integer unless t lies within 1e-4 of a
-// half-integer; only then is the quotient formed exactly.  The rounding itself is done by adding
-// 1.5 * 2^23 (round-to-nearest-even puts the integer in the low mantissa bits, so the low byte of the
-// sum IS the two's-complement INT8 code).  Eight elements at a time, packed FP32x2 arithmetic; the
-// distance of every t from its rounded value is folded into the running maximum `dmax`, which the caller
-// checks (once per vector or once per several): above kQuantTieGuard some element is (nearly) a tie and
-// quant8_exact has to be used instead.
-constexpr float kQuantTieGuard = 0.4999f;
-
-__device__ __forceinline__ uint2 quant8_fast(const uint4& v, float rdelta, float& dmax) {
+// Eight elements, packed FP32x2 arithmetic.
+template <bool REFINE>
+__device__ __forceinline__ uint2 quant8(const uint4& v, const QuantScale& s) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    const float2 r2 = make_float2(rdelta, rdelta);
-    const float2 magic = make_float2(12582912.f, 12582912.f), nmagic = make_float2(-12582912.f, -12582912.f);
+    const float2 r2 = make_float2(s.r, s.r), nd2 = make_float2(-s.delta, -s.delta);
+    const float2 magic = make_float2(12582912.f, 12582912.f);
     float2 y[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const float2 x = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-        const float2 t = __fmul2_rn(x, r2);
-        y[i] = __fadd2_rn(t, magic);
-        const float2 back = __fadd2_rn(y[i], nmagic);
-        const float2 d = __fadd2_rn(t, make_float2(-back.x, -back.y));
-        dmax = fmaxf(dmax, fmaxf(fabsf(d.x), fabsf(d.y)));
+        if constexpr (REFINE) {
+            float2 q = __fmul2_rn(x, r2);
+            q = __ffma2_rn(__ffma2_rn(nd2, q, x), r2, q);
+            y[i] = __fadd2_rn(q, magic);
+        } else {
+            y[i] = __ffma2_rn(x, r2, magic);
+        }
     }
     // low bytes of the eight sums -> two words
     const uint32_t p0 = __byte_perm(__float_as_uint(y[0].x), __float_as_uint(y[0].y), 0x0040);
@@ -51,54 +70,8 @@ __device__ __forceinline__ uint2 quant8_fast(const uint4& v, float rdelta, float
     const uint32_t p3 = __byte_perm(__float_as_uint(y[3].x), __float_as_uint(y[3].y), 0x0040);
     return make_uint2(__byte_perm(p0, p1, 0x5410), __byte_perm(p2, p3, 0x5410));
 }
-
-// The definition, element by element.
-__device__ __forceinline__ uint2 quant8_exact(const uint4& v, float delta) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint32_t o[2] = {0u, 0u};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 x = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-        const uint32_t lo = static_cast<uint32_t>(quant1_exact(x.x, delta)) & 0xffu;
-        const uint32_t hi = static_cast<uint32_t>(quant1_exact(x.y, delta)) & 0xffu;
-        o[i >> 1] |= (lo | (hi << 8)) << ((i & 1) * 16);
-    }
-    return make_uint2(o[0], o[1]);
-}
-
-// Branch-free form for a caller whose lanes must not diverge (the attention kernel's on-chip quantiser):
-// the IEEE quotient itself, by the classical refinement with the exact residual -- q0 = x * r with
-// r = RN(1/delta), then twice q <- q + (x - delta * q) * r, the residual being exact in one FMA.  The first
-// step leaves q within one unit in the last place of x / delta, the second rounds it correctly (the final
-// step of a software division; no operand here is near the underflow or overflow range: |x| is a
-// binary16 magnitude, |x / delta| <= 127.5).  The integer rounding is the magic-number add of quant8_fast.
-__device__ __forceinline__ uint2 quant8_div(const uint4& v, float delta, float rdelta) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    const float2 r2 = make_float2(rdelta, rdelta), nd2 = make_float2(-delta, -delta);
-    const float2 magic = make_float2(12582912.f, 12582912.f);
-    float2 y[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 x = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-        float2 q = __fmul2_rn(x, r2);
-        float2 e = __ffma2_rn(nd2, q, x);
-        q = __ffma2_rn(e, r2, q);
-        e = __ffma2_rn(nd2, q, x);
-        q = __ffma2_rn(e, r2, q);
-        y[i] = __fadd2_rn(q, magic);
-    }
-    const uint32_t p0 = __byte_perm(__float_as_uint(y[0].x), __float_as_uint(y[0].y), 0x0040);
-    const uint32_t p1 = __byte_perm(__float_as_uint(y[1].x), __float_as_uint(y[1].y), 0x0040);
-    const uint32_t p2 = __byte_perm(__float_as_uint(y[2].x), __float_as_uint(y[2].y), 0x0040);
-    const uint32_t p3 = __byte_perm(__float_as_uint(y[3].x), __float_as_uint(y[3].y), 0x0040);
-    return make_uint2(__byte_perm(p0, p1, 0x5410), __byte_perm(p2, p3, 0x5410));
-}
-
-__device__ __forceinline__ uint2 quant8(const uint4& v, float delta, float rdelta) {
-    float dmax = 0.f;
-    const uint2 q = quant8_fast(v, rdelta, dmax);
-    if (dmax > kQuantTieGuard) return quant8_exact(v, delta);
-    return q;
+__device__ __forceinline__ uint2 quant8(const uint4& v, const QuantScale& s) {
+    return s.refine ? quant8<true>(v, s) : quant8<false>(v, s);
 }
 
 }  // namespace tilemix

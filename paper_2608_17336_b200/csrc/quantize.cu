@@ -78,9 +78,8 @@ quantize_kernel(const __half* __restrict__ x, int64_t s_batch, int64_t s_head, i
     for (int w = 0; w < kThreads / 32; ++w) amax = max(amax, warp_max[w]);
 
     const float amax_f = __half2float(__ushort_as_half(static_cast<unsigned short>(amax)));
-    const float delta = __fdiv_rn(amax_f, 127.0f);
-    const float rdelta = __frcp_rn(delta);
-    if (threadIdx.x == 0) scale[scale_idx] = delta;
+    const QuantScale qs = quant_scale(amax_f);
+    if (threadIdx.x == 0) scale[scale_idx] = qs.delta;
 
     if (amax == 0u) {  // zero block: delta = 0, xhat = 0 (no division by zero)
         for (int v = threadIdx.x; v < nvec; v += kThreads)
@@ -90,12 +89,12 @@ quantize_kernel(const __half* __restrict__ x, int64_t s_batch, int64_t s_head, i
 #pragma unroll
     for (int i = 0; i < MAXV; ++i) {
         const int v = threadIdx.x + i * kThreads;
-        if (v < nvec) *reinterpret_cast<uint2*>(dst + static_cast<int64_t>(v) * 8) = quant8(cache[i], delta, rdelta);
+        if (v < nvec) *reinterpret_cast<uint2*>(dst + static_cast<int64_t>(v) * 8) = quant8(cache[i], qs);
     }
     for (int v = threadIdx.x + MAXV * kThreads; v < nvec; v += kThreads) {
         const int row = v / vec_per_row, c8 = v - row * vec_per_row;
         const uint4 t = __ldg(reinterpret_cast<const uint4*>(src + row * s_tok + c8 * 8));
-        *reinterpret_cast<uint2*>(dst + static_cast<int64_t>(v) * 8) = quant8(t, delta, rdelta);
+        *reinterpret_cast<uint2*>(dst + static_cast<int64_t>(v) * 8) = quant8(t, qs);
     }
 }
 
@@ -217,15 +216,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) quantize_stream_kernel(cons
 #pragma unroll
             for (int x = 0; x < kStreamWarps; ++x) amax = max(amax, warp_max[grp][par][x]);
             const float amax_f = __half2float(__ushort_as_half(static_cast<unsigned short>(amax)));
-            const float delta = __fdiv_rn(amax_f, 127.0f);
-            const float rdelta = __frcp_rn(delta);
-            if (gtid == 0) *w.scale = delta;
+            QuantScale qs = quant_scale(amax_f);
+            if (gtid == 0) *w.scale = qs.delta;
+            if (amax == 0u) qs.r = 0.f, qs.refine = false;      // zero block: delta = 0, xhat = 0
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int v = gtid + i * (kStreamWarps * 32);
-                if (v < nvec)
-                    *reinterpret_cast<uint2*>(w.dst + static_cast<int64_t>(v) * 8) =
-                        amax == 0u ? make_uint2(0u, 0u) : quant8(cache[i], delta, rdelta);   // zero block: delta = 0, xhat = 0
+                if (v < nvec) *reinterpret_cast<uint2*>(w.dst + static_cast<int64_t>(v) * 8) = quant8(cache[i], qs);
             }
             done = t + kStreamGroups;      // (this group's next block)
         }
