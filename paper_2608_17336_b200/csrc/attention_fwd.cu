@@ -1258,6 +1258,12 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
 
 }  // namespace
 
+int encode_rows_map(CUtensorMap* tm, const void* base, int d, int L, int H, int B, const int64_t stride_elems[3], int box_rows) {
+    EncodeTiledFn enc = nullptr;
+    const int rc = get_encoder(&enc);
+    return rc ? rc : encode_map(enc, tm, base, 2, d, L, H, B, stride_elems, d, box_rows, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
 int launch_attention(const Geometry& g, const void* q, const void* k, const void* v, const int8_t* q8,
                      const int8_t* k8, const float* qs, const float* ks, const uint32_t* words, void* out,
                      float* lse, void* workspace, const tilemix_debug_t* dbg, cudaStream_t stream,

@@ -2,6 +2,7 @@
 // resolved geometry, launch counting).  Not part of the public ABI.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -88,7 +89,10 @@ int launch_quantize(const void* x, const int64_t stride[3], int B, int H, int L,
                     const int32_t* blk_off = nullptr, int total_blk = 0);
 int launch_quantize_pair(const void* q, const int64_t qstride[3], int Hq, int blk_q, int8_t* q8, float* qs,
                          const void* k, const int64_t kstride[3], int Hk, int blk_k, int8_t* k8, float* ks,
-                         int B, int L, int d, cudaStream_t stream);
+                         int B, int L, int d, cudaStream_t stream, const VarlenDev* vl = nullptr,
+                         int total_blk_q = 0, int total_blk_k = 0);
+// Tensor map over an FP16 [B, H, L, d] operand whose box is box_rows whole rows, unswizzled (attention_fwd.cu).
+int encode_rows_map(CUtensorMap* tm, const void* base, int d, int L, int H, int B, const int64_t stride_elems[3], int box_rows);
 int launch_pack(const Geometry& g, const uint8_t* route, uint32_t pack_flags, uint32_t* words,
                 unsigned long long* counts, cudaStream_t stream, const VarlenDev* vl = nullptr);
 int launch_attention(const Geometry& g, const void* q, const void* k, const void* v,

@@ -146,6 +146,9 @@ int tilemix_quantize_qk_varlen(const tilemix_problem_t* p, const tilemix_varlen_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     VarlenDev dev;
     if ((rc = upload_varlen(t, workspace, s, &dev))) return rc;
+    if (do_q && do_k)
+        return launch_quantize_pair(q_f16, g.qs, g.Hq, g.blk_q, q_i8, q_scale, k_f16, g.ks, g.Hk, g.blk_k, k_i8, k_scale, 1, g.L, g.d,
+                                    s, &dev, t.total_blk_q, t.total_blk_k);
     if (do_q && t.total_blk_q > 0 &&
         (rc = launch_quantize(q_f16, g.qs, 1, g.Hq, g.L, g.d, g.blk_q, q_i8, q_scale, s, &dev, dev.blkq, t.total_blk_q)))
         return rc;
