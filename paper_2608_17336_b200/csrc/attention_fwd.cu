@@ -463,6 +463,13 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         return a == 0.f ? -1.f : -a;
     };
 
+    // On-the-fly mode: the chunks are not a ring but fixed places -- V in chunks 0-1, the FP16 copy of key tile n in 2-3 or
+    // 4-5 and its INT8 copy in 6 or 7 by the parity of n -- so that the next FP16 tile is on its way while the quantiser
+    // works on this one.  (In the ring, where V, K16 and K8 of 80 KB per key tile follow one another, it could only be
+    // asked for when the tile before had been consumed: 3640 of 6800 clk per key tile were spent waiting for it.)
+    auto otf_k16 = [](int n) -> uint32_t { return 2u + 2u * (n & 1); };
+    auto otf_k8 = [](int n) -> uint32_t { return 6u + (n & 1); };
+
     if (OTF && warp >= kQuantWarp0) {
         // ================================================================ on-chip quantiser (on-the-fly mode)
         // Four warps make the INT8 copies the tensor pipe reads: of a query tile before the first key tile it
@@ -545,15 +552,11 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         // The quantiser arrives on the "landed" barrier of EVERY bundle, with or without an INT8 tile to
         // make, so that the issuers (and with them the producer) can never run more than kBundles bundles
         // ahead of it and the phase it waits for is unambiguous.
-        Ring ring;   // the producer's sequence of chunks
         uint32_t q8_made = 0u;
         volatile float* dq_s = reinterpret_cast<volatile float*>(misc + 12);   // delta_Q of the two query tiles
         for (int n = 0; n < nkv; ++n) {
             const uint32_t e = sched(n);
-            uint32_t s16 = 0, s8 = 0;
-            if (n >= 1) ring.take(C::kHalves);
-            if (e & kNeed16) s16 = ring.take(C::kHalves);
-            if (e & kNeed8) s8 = ring.take(1);
+            const uint32_t s16 = otf_k16(n), s8 = otf_k8(n);
             for (int t = 0; t < 2; ++t) {
                 if (!((e >> t) & 1u) || ((q8_made >> t) & 1u)) continue;
                 if (ok) ok = wait_bar(cx, bar_q(t), 0, kRoleQuant, t, kBarQ);
@@ -668,9 +671,9 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 // quantiser (bar_raw), not to the issuers; the INT8 chunk is only claimed, not filled.
                 const bool make8 = OTF && (e & kNeed8);
                 // chunk order inside the sequence: ..., V_{n-1}, K16_n, K8_n, V_n, ...
-                if (has_v) { sv = ring.take(C::kHalves); bytes += C::kHalves * C::kChunk; }
-                if (e & kNeed16) { s16 = ring.take(C::kHalves); (make8 ? raw_bytes : bytes) += C::kHalves * C::kChunk; }
-                if (e & kNeed8) { s8 = ring.take(1); if (!OTF) bytes += C::kK8Bytes; }
+                if (has_v) { sv = OTF ? 0u : ring.take(C::kHalves); bytes += C::kHalves * C::kChunk; }
+                if (e & kNeed16) { s16 = OTF ? otf_k16(n) : ring.take(C::kHalves); (make8 ? raw_bytes : bytes) += C::kHalves * C::kChunk; }
+                if (e & kNeed8) { s8 = OTF ? otf_k8(n) : ring.take(1); if (!OTF) bytes += C::kK8Bytes; }
                 if (bytes == 0u && raw_bytes == 0u) break;             // nothing after the last V
                 if (n == prm.test_drop_bundle) {   // testing aid: this bundle never lands, an issuer's bounded wait runs out
                     dropped = n;
@@ -697,26 +700,37 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         last_user[slot + c] = n;
                     }
                 };
-                if (has_v) {
-                    claim(sv, C::kHalves);
-                    if (!ok) break;
+                auto load_v = [&]() {
                     for (int c = 0; c < C::kHalves; ++c)
                         ptx::tma_load_4d(sbase + C::kOffRing + (sv + c) * C::kChunk, &tm_v16, bar, c * 64, tok0 + (n - 1) * T, hk, b);
+                };
+                if (has_v && !OTF) {
+                    claim(sv, C::kHalves);
+                    if (!ok) break;
+                    load_v();
                 }
+                // on-the-fly mode: K first, into the places of key tile n - 2; V behind it, when V of key tile n - 2 is done with
+                if (OTF && n >= 2) wait_consumed(n - 2, n);
+                if (!ok) break;
                 if (e & kNeed16) {
-                    claim(s16, C::kHalves);
+                    if (!OTF) claim(s16, C::kHalves);
                     if (!ok) break;
                     const uint32_t bar16 = make8 ? bar_raw(n % kBundles) : bar;
                     for (int c = 0; c < C::kHalves; ++c)
                         ptx::tma_load_4d(sbase + C::kOffRing + (s16 + c) * C::kChunk, &tm_k16, bar16, c * 64, tok0 + n * T, hk, b);
                 }
-                if (e & kNeed8) {
+                if (!OTF && (e & kNeed8)) {
                     claim(s8, 1);
                     if (!ok) break;
-                    if (!OTF) ptx::tma_load_4d(sbase + C::kOffRing + s8 * C::kChunk, &tm_k8, bar, 0, tok0 + n * T, hk, b);
+                    ptx::tma_load_4d(sbase + C::kOffRing + s8 * C::kChunk, &tm_k8, bar, 0, tok0 + n * T, hk, b);
                 }
                 // on-the-fly mode, second arrival: the INT8 chunk (if any) is the quantiser's to write
                 if (OTF && n < nkv) ptx::mbar_arrive(bar_raw(n % kBundles));
+                if (has_v && OTF) {
+                    wait_consumed(n - 1, n);
+                    if (!ok) break;
+                    load_v();
+                }
             }
             if (!ok || *cx.abort_flag) {
                 // let copies that are still in flight land before the CTA's memory is released
@@ -838,8 +852,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             uint32_t e_next = sched(0), k16 = 0, k8 = 0;
             // route of this tile at half h of the key tile of entry e (D = 64: bits 0 / 1 = the two row halves)
             auto route = [&](uint32_t e, int h) -> uint32_t { return SUB ? (e >> (4 * h + 2 * t)) & 3u : (e >> t) & 1u; };
-            if (e_next & kNeed16) k16 = ring.take(C::kHalves);
-            if (e_next & kNeed8) k8 = ring.take(1);
+            if (e_next & kNeed16) k16 = OTF ? otf_k16(0) : ring.take(C::kHalves);
+            if (e_next & kNeed8) k8 = OTF ? otf_k8(0) : ring.take(1);
             acquire(0);
             if (ok) {
                 ptx::tc_fence_after_sync();
@@ -852,10 +866,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             }
             for (int j = 0; j < nkv && ok; ++j) {
                 const bool mine = 2 * j < u_t;         // tile A has no work at the last key tile of tile B
-                const uint32_t sv = ring.take(C::kHalves);
+                const uint32_t sv = OTF ? 0u : ring.take(C::kHalves);
                 e_next = (j + 1 < nkv) ? sched(j + 1) : 0u;
-                if (e_next & kNeed16) k16 = ring.take(C::kHalves);
-                if (e_next & kNeed8) k8 = ring.take(1);
+                if (e_next & kNeed16) k16 = OTF ? otf_k16(j + 1) : ring.take(C::kHalves);
+                if (e_next & kNeed8) k8 = OTF ? otf_k8(j + 1) : ring.take(1);
                 // operands of this iteration (bundle j + 1): wait for them now, off the P -> PV critical path
                 acquire(j + 1);
                 if (!ok) break;
