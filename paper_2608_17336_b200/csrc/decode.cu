@@ -3,7 +3,7 @@
 // HBM-bound: a cached token costs d bytes of K8 (or 2d of FP16 K on the FP16 route) plus d bytes of
 // V8, each read once.  This file holds the host entry points, the preparation and merge kernels, and the
 // warp-level form of the step for head_dim 64 or 64-key tiles: the tiles are streamed into a shared-memory
-// ring by untiled bulk copies, a tile ahead of their use, and the H_q/H_k query rows of a KV head are the
+// ring by untiled bulk copies, and the H_q/H_k query rows of a KV head are the
 // rows of a 16-row warp-level tensor-core operand.  head_dim 128 with 128-key tiles runs the tcgen05 form
 // (decode_umma.cu), where the KEYS are the MMA rows.
 #include <cuda_fp16.h>
@@ -21,16 +21,77 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 
-constexpr int kStages = 2;    // ring of key/value tiles in shared memory when FP16 keys may be read ...
-constexpr int kStagesInt8 = 3;   // ... and when there is no FP16 key cache (a stage is a third smaller)
-constexpr int kChunk = 128;   // keys per kernel tile when tile_n allows it (64-key tiles with deeper rings were slower)
+// Keys per kernel tile.  Head dimension 64: 128, i.e. one routing tile of 128 keys or two of 64 (each of the eight warps
+// has a 16-key step of its own).  Head dimension 128 (64-key routing tiles): 64, two warps per step with half of the
+// output columns each; a warp with all 128 columns needs more than its 128 registers (8 x 16K keys: 97 us, 118 that way).
+template <int D>
+constexpr int kChunk = D == 64 ? 128 : 64;
 
-template <int D, int T>
+// Ring of kernel tiles in shared memory.  What bounds the step is the data in flight: two CTAs per SM with 96 KB each keep
+// what the HBM latency asks for on the way (two stages before, 24 KB with 64-key tiles of dimension 64; that, two such
+// tiles per kernel tile and the shares below: 16 sequences of up to 8K keys, 32 / 8 heads of 64, 67 -> 42 us).
+constexpr int kRingBytes = 96 * 1024;
+template <int D, bool F16K>
 struct Stage {
-    static constexpr int kK = T * D * 2;   // room for the FP16 copy of a key tile
-    static constexpr int kV = T * D;
+    static constexpr int kK = kChunk<D> * D * (F16K ? 2 : 1);   // room for the FP16 copy of the keys, if there is one
+    static constexpr int kV = kChunk<D> * D;
     static constexpr int kBytes = kK + kV;
+    static constexpr int kStages = kRingBytes / kBytes;
 };
+constexpr int kMaxStages = 6;
+
+// Rows of unequal cache lengths (the library chooses the splits): the `pool` partial results that a KV head's workspace
+// has room for are shared out over the sequences by their length, s_b = max(1, ceil(tiles_b / q)) CTAs to sequence b for
+// the smallest q whose total fits, so that the CTAs of the grid finish together.  Lane l of a warp works on sequences
+// l * K .. l * K + K - 1 (K = ceil(B / 32) <= kShareRows); every warp that asks finds the same shares.
+constexpr int kShareRows = 8, kMaxShared = 32 * kShareRows;
+struct Shares {
+    int s[kShareRows];   // CTAs of this lane's sequences
+    int start;           // first CTA of the lane's first sequence
+    int K;
+};
+template <int T>
+__device__ __forceinline__ Shares share_out(const int32_t* __restrict__ cache_len, int B, int max_len, int pool) {
+    const int lane = threadIdx.x & 31;
+    Shares sh;
+    sh.K = (B + 31) >> 5;
+    int tiles[kShareRows], total = 0, longest = 1;
+#pragma unroll
+    for (int k = 0; k < kShareRows; ++k) {
+        const int b = lane * sh.K + k;
+        tiles[k] = k < sh.K && b < B ? (min(max(cache_len[b], 0), max_len) + T - 1) / T : -1;
+        total += max(tiles[k], 0);
+        longest = max(longest, tiles[k]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        total += __shfl_xor_sync(0xffffffffu, total, o);
+        longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, o));
+    }
+    auto share = [&](int t, int q) -> int { return t < 0 ? 0 : max(1, (t + q - 1) / q); };
+    int lo = max(1, (total + pool - 1) / pool);
+    int hi = pool > B ? max(lo, min(longest, (total + pool - B - 1) / (pool - B))) : max(lo, longest);   // fits: sum of ceil(t / q) <= total / q + B
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < kShareRows; ++k) n += share(tiles[k], mid);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+        if (n <= pool) hi = mid; else lo = mid + 1;
+    }
+    int mine = 0;
+#pragma unroll
+    for (int k = 0; k < kShareRows; ++k) { sh.s[k] = share(tiles[k], hi); mine += sh.s[k]; }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    sh.start = incl - mine;
+    return sh;
+}
 
 // ---- warp-level tensor-core MMAs (m16n8k32 INT8 / m16n8k16 FP16, FP32 or INT32 accumulators) ----------
 // Lane l holds, with g = l / 4 and t = l % 4: A rows g (a0, a2) and g + 8 (a1, a3), B column g, C rows g
@@ -47,12 +108,11 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a2,
                  : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
 }
 
-// D: head dim; R: query heads per KV head; T: keys per tile (= scale block = routing tile).
+// D: head dim; R: query heads per KV head; RT: keys per routing tile (= scale block); a kernel tile is T keys.
 // Tiles are contiguous in the cache, so they are streamed into a ring of shared-memory stages with
 // untiled bulk copies ("full" / "empty" mbarriers per stage), issued by one lane of the last warp
 // before it turns to its own share of a tile.  The eight warps never synchronise with one another
-// inside the loop: each one owns 16 keys of every tile (and, for
-// 64-key tiles, half of the output columns) and runs its own flash-decoding recurrence on them --
+// inside the loop: each one owns 16 keys of every tile and runs its own flash-decoding recurrence on them --
 //  (1) scores S[R x 16] = Q K^T on the tensor cores, the R query rows being rows 0..R-1 of a 16-row A
 //      operand.  The contraction index may be permuted freely as long as Q and K use the same
 //      permutation, so lane t simply takes the 16-byte chunks t, t+4, ... of a row;
@@ -65,36 +125,53 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a2,
 constexpr int kConsumerWarps = 8;
 constexpr int kDecodeThreads = kConsumerWarps * 32;   // 2 CTAs/SM = 4 warps per scheduler: 128 registers each
 
-template <int D, int R, int T, bool F16K>
+template <int D, int R, int RT, bool F16K>
 __global__ void __launch_bounds__(kDecodeThreads, 2)
 decode_kernel(const DecodeParams prm) {
-    using St = Stage<D, T>;
+    constexpr int T = kChunk<D>, SUBN = T / RT;   // routing tiles of a kernel tile
+    using St = Stage<D, F16K>;
     constexpr int W8 = D / 16, W16 = D / 8;       // 32-bit words per lane and row: INT8 / FP16 operand
     constexpr int KS3 = T / 16;                   // 16-key steps of a tile
     constexpr int NSPLIT = kConsumerWarps / KS3;  // warps sharing one step (each takes some column blocks)
-    constexpr int NBLK = D / 8 / NSPLIT;          // column blocks per warp
+    constexpr int NBLK = D / 8 / NSPLIT;          // column blocks of 8 per warp
     constexpr int BPG = D / 8;                    // bytes of a cached V row per lane group
     static_assert(KS3 <= kConsumerWarps && kConsumerWarps % KS3 == 0, "tile shape vs warps");
-    static_assert(kStagesInt8 * 2 * St::kV >= static_cast<int>(kConsumerWarps * R * (D + 2) * sizeof(float)),
-                  "the final merge reuses the ring");
-    const int split = blockIdx.x, hk = blockIdx.y, b = blockIdx.z;
+    static_assert(kRingBytes >= static_cast<int>(kConsumerWarps * R * (D + 2) * sizeof(float)), "the final merge reuses the ring");
+    static_assert(St::kStages <= kMaxStages, "barriers of the ring");
+    const int hk = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t = lane & 3;
-    // (lengths live on the device and cannot be checked by the host: out-of-range values are clamped)
-    const int len = prm.cache_len[b];   // the clamped copy decode_prepare_kernel made
+    int split = blockIdx.x, b = blockIdx.z, row_splits = prm.n_splits;
+    if (prm.balanced) {      // gridDim.x CTAs per KV head, shared out over the sequences
+        const Shares sh = share_out<T>(prm.cache_len_raw, prm.B, prm.max_len, prm.n_ctas);
+        int found = -1, part = 0, n = 0, start = sh.start;
+#pragma unroll
+        for (int k = 0; k < kShareRows; ++k) {
+            const int at = static_cast<int>(blockIdx.x) - start;
+            if (at >= 0 && at < sh.s[k]) { found = lane * sh.K + k; part = at; n = sh.s[k]; }
+            start += sh.s[k];
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, found >= 0);
+        if (who == 0u) return;                                    // a CTA left over
+        const int src = __ffs(who) - 1;
+        b = __shfl_sync(0xffffffffu, found, src);
+        split = __shfl_sync(0xffffffffu, part, src);
+        row_splits = __shfl_sync(0xffffffffu, n, src);
+    }
+    // (lengths live on the device and cannot be checked by the host: out-of-range values are clamped.  This grid may run
+    // beside the prepare kernel, so it clamps the caller's array itself, and waits for that kernel only where it writes
+    // the status record.)
+    const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
-    const int per_split = (n_tiles + prm.n_splits - 1) / prm.n_splits;
+    const int per_split = (n_tiles + row_splits - 1) / row_splits;
     const int t0 = split * per_split, t1 = min(n_tiles, t0 + per_split);
 
     extern __shared__ __align__(128) uint8_t ring[];   // n_stages x (K tile | V tile)
-    // without an FP16 key cache a K slot only ever holds INT8 keys: smaller stages, one more of them
-    constexpr int n_stages = F16K ? kStages : kStagesInt8;
-    constexpr int k_slot = F16K ? St::kK : St::kV;
-    constexpr int stage_bytes = k_slot + St::kV;
+    constexpr int n_stages = St::kStages, k_slot = St::kK, stage_bytes = St::kBytes;
     __shared__ __align__(16) uint32_t qh[R][D / 2];   // query rows, FP16 pairs (FP16 route)
     __shared__ __align__(16) uint32_t q8w[R][D / 4];  // quantised query rows, 4 bytes per word (INT8 route)
     __shared__ float dq_s[R];
-    __shared__ __align__(8) uint64_t full_bar[kStagesInt8], empty_bar[kStagesInt8];
+    __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
     __shared__ int abort_flag;
     // route bit (sign) and the two block scales of the first kMetaTiles tiles of this split, staged once
     constexpr int kMetaTiles = 256;
@@ -102,7 +179,7 @@ decode_kernel(const DecodeParams prm) {
 
     const uint32_t ring_u32 = ptx::smem_u32(ring);
     if (tid == 0) {
-        for (int s = 0; s < kStagesInt8; ++s) {
+        for (int s = 0; s < n_stages; ++s) {
             ptx::mbar_init(ptx::smem_u32(&full_bar[s]), 1);
             ptx::mbar_init(ptx::smem_u32(&empty_bar[s]), kConsumerWarps);
         }
@@ -145,11 +222,9 @@ decode_kernel(const DecodeParams prm) {
     const float* dv = prm.v_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.n_blk;
     const uint32_t* wrow = prm.words != nullptr
         ? prm.words + (static_cast<int64_t>(prm.nb == 1 ? 0 : b) * prm.Hk + hk) * prm.W : nullptr;
-    // the kernel's tile (T keys) may be a fraction of the scale block / routing tile tile_n
-    const int per_blk = prm.tile_n / T;
-    auto route_of = [&](int tile) -> bool {
+    auto route_of = [&](int rt) -> bool {      // of a routing tile
         if (wrow == nullptr) return false;
-        const int grp = tile / (per_blk * prm.G);
+        const int grp = rt / prm.G;
         return (wrow[grp >> 5] >> (grp & 31)) & 1u;
     };
     // Bounded wait on a ring barrier; false when the CTA is giving up.
@@ -169,18 +244,21 @@ decode_kernel(const DecodeParams prm) {
         }
         return true;
     };
-    for (int i = tid; i < kMetaTiles && t0 + i < t1; i += kDecodeThreads) {
-        const int tile = t0 + i;
+    // routing tiles of this split (the last kernel tile of a row may have one only)
+    const int rt0 = t0 * SUBN, rt1 = min(t1 * SUBN, (len + RT - 1) / RT);
+    for (int i = tid; i < kMetaTiles && rt0 + i < rt1; i += kDecodeThreads) {
+        const int rt = rt0 + i;
         // delta_K >= 0; the FP16 route is marked by a negative x (its delta_K is not used)
-        meta[i] = make_float2(route_of(tile) ? dk[tile / per_blk] : -1.f, dv[tile / per_blk]);
+        meta[i] = make_float2(route_of(rt) ? dk[rt] : -1.f, dv[rt]);
     }
     if constexpr (!F16K) {
         // This instance was chosen because no FP16 key cache was passed: every group inside the cache length has
         // to be INT8-routed.  A 0 bit is found here, before any copy is started; the CTA records it and leaves
         // (no access is made, nothing is in flight).
         int fp16_group = 0;
-        for (int tile = t0 + tid; tile < t1; tile += kDecodeThreads) fp16_group |= route_of(tile) ? 0 : 1;
+        for (int rt = rt0 + tid; rt < rt1; rt += kDecodeThreads) fp16_group |= route_of(rt) ? 0 : 1;
         if (__syncthreads_or(fp16_group)) {
+            ptx::griddep_wait();
             if (tid == 0 && atomicCAS(&prm.status[0], 0, TILEMIX_ERR_NULL) == 0) {
                 prm.status[1] = 16; prm.status[2] = t0; prm.status[3] = 1;
             }
@@ -189,6 +267,7 @@ decode_kernel(const DecodeParams prm) {
     } else {
         __syncthreads();   // barriers initialised, query rows and tile metadata staged
     }
+    ptx::griddep_launch_dependents();     // the merge kernel may be brought in; it waits for this grid to finish
 
     // per-warp flash-decoding state: rows g (< R) of this warp's keys
     float m_run = -INFINITY, z_part = 0.f;          // z_part: this lane's share of the row sum
@@ -207,25 +286,42 @@ decode_kernel(const DecodeParams prm) {
         if (it == prm.test_drop_tile) return true;   // testing aid: this tile never lands, the consumers' bounded wait runs out
         // the first pass over the ring finds every stage free
         if (it >= n_stages && !wait_ring(&empty_bar[stage], ((it / n_stages) - 1) & 1)) return false;
-        const uint32_t rows = static_cast<uint32_t>(min(T, len - tile * T));   // only rows that exist
+        const int rows = min(T, len - tile * T);   // only rows that exist
         const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
         const uint32_t dst = ring_u32 + stage * stage_bytes;
-        const bool int8 = route_of(tile);
-        const uint32_t kbytes = rows * D * (int8 ? 1u : 2u);
-        ptx::mbar_arrive_expect_tx(bar, kbytes + rows * D);
-        if (int8) ptx::bulk_load_1d(dst, k8 + static_cast<int64_t>(tile) * T * D, kbytes, bar);
-        else ptx::bulk_load_1d(dst, k16 + static_cast<int64_t>(tile) * T * D, kbytes, bar);
+        uint32_t kbytes[SUBN], bytes = rows * D;
+        bool int8[SUBN];
+#pragma unroll
+        for (int i = 0; i < SUBN; ++i) {
+            const int r = max(0, min(RT, rows - i * RT));
+            int8[i] = r > 0 && route_of(tile * SUBN + i);
+            kbytes[i] = r * D * (int8[i] ? 1 : 2);
+            bytes += kbytes[i];
+        }
+        ptx::mbar_arrive_expect_tx(bar, bytes);
+#pragma unroll
+        for (int i = 0; i < SUBN; ++i) {
+            const int64_t at = static_cast<int64_t>(tile * SUBN + i) * RT * D;
+            const uint32_t kdst = dst + i * (k_slot / SUBN);
+            if (kbytes[i] == 0u) continue;
+            if (int8[i]) ptx::bulk_load_1d(kdst, k8 + at, kbytes[i], bar);
+            else ptx::bulk_load_1d(kdst, k16 + at, kbytes[i], bar);
+        }
         ptx::bulk_load_1d(dst + k_slot, v8 + static_cast<int64_t>(tile) * T * D, rows * D, bar);
         last_produced = tile;
         return true;
     };
     const bool producer = warp == kConsumerWarps - 1 && lane == 0;
+    // tiles asked for ahead of the one in work: with a deep ring one less than fits, so that the producing warp does
+    // not wait for the slowest warp to hand back the tile it has itself just finished
+    constexpr int kAhead = n_stages > 3 ? n_stages - 2 : n_stages - 1;
     if (producer)
-        for (int s = 0; s < n_stages - 1 && t0 + s < t1; ++s) produce(t0 + s);
+        for (int s = 0; s < kAhead && t0 + s < t1; ++s) produce(t0 + s);
     {
         // ================================================================ consumers
-        const int ks = warp / NSPLIT, nb0 = (warp % NSPLIT) * NBLK;   // this warp's keys and column blocks
+        const int ks = warp / NSPLIT, nb0 = (warp % NSPLIT) * NBLK;   // this warp's keys (16 ks ..) and column blocks
         const bool counts_z = (warp % NSPLIT) == 0;                    // one warp per key step sums z
+        const int sub = 16 * ks / RT, key_in_rt = 16 * ks - sub * RT;  // the keys' routing tile of the kernel tile
         // A fragments of the INT8 route: lane t's words of query row g, in the order the K words are used
         uint32_t qa8[W8];
 #pragma unroll
@@ -234,30 +330,34 @@ decode_kernel(const DecodeParams prm) {
 
         for (int tile = t0; tile < t1; ++tile) {
             const int it = tile - t0, stage = it % n_stages;
-            if (producer && tile + n_stages - 1 < t1) produce(tile + n_stages - 1);   // keeps the ring full
+            if (producer && tile + kAhead < t1) produce(tile + kAhead);   // keeps the ring full
             // route bit and block scales: from shared memory (global loads for tiles beyond the staged ones)
             bool int8;
             float dkt, dvt;
-            if (it < kMetaTiles) {
-                const float2 mt = meta[it];
+            const int rt = tile * SUBN + sub;
+            if (rt >= rt1) {               // (no such keys: all are masked below)
+                int8 = true;
+                dkt = dvt = 0.f;
+            } else if (rt - rt0 < kMetaTiles) {
+                const float2 mt = meta[rt - rt0];
                 int8 = mt.x >= 0.f;
                 dkt = mt.x;
                 dvt = mt.y;
             } else {
-                int8 = route_of(tile);
-                dkt = int8 ? dk[tile / per_blk] : 0.f;
-                dvt = dv[tile / per_blk];
+                int8 = route_of(rt);
+                dkt = int8 ? dk[rt] : 0.f;
+                dvt = dv[rt];
             }
             if (!wait_ring(&full_bar[stage], (it / n_stages) & 1)) break;
-            const uint8_t* kst = ring + stage * stage_bytes;
-            const uint8_t* vst = kst + k_slot;
+            const uint8_t* vst = ring + stage * stage_bytes + k_slot;
+            const uint8_t* kst = ring + stage * stage_bytes + sub * (k_slot / SUBN);
             // ---- (1) scores of this warp's 16 keys, rows g: s[nb][0..1] = keys 8 nb + 2t, 2t + 1 ----------
             float sc[2][2];
             if (int8) {
                 const float a = prm.scale_log2 * dq * dkt;
 #pragma unroll
                 for (int nb = 0; nb < 2; ++nb) {
-                    const uint8_t* krow = kst + (16 * ks + 8 * nb + g) * D;       // B column g = that key
+                    const uint8_t* krow = kst + (key_in_rt + 8 * nb + g) * D;       // B column g = that key
                     uint32_t kw[W8];
 #pragma unroll
                     for (int ch = 0; ch < W8 / 4; ++ch) {
@@ -280,7 +380,7 @@ decode_kernel(const DecodeParams prm) {
                 }
 #pragma unroll
                 for (int nb = 0; nb < 2; ++nb) {
-                    const uint8_t* krow = kst + (16 * ks + 8 * nb + g) * D * 2;
+                    const uint8_t* krow = kst + (key_in_rt + 8 * nb + g) * D * 2;
                     float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int ch = 0; ch < W16 / 4; ++ch) {
@@ -367,6 +467,7 @@ decode_kernel(const DecodeParams prm) {
     // ---- merge of the eight warps, then (m, z, O~) of this split to the workspace --------------------
     __syncthreads();   // every warp is out of the ring (all copies it waited for have landed)
     if (*reinterpret_cast<volatile int*>(&abort_flag)) {
+        ptx::griddep_wait();
         if (tid == 0 && atomicCAS(&prm.status[0], 0, TILEMIX_ERR_DEVICE_TIMEOUT) == 0) {
             prm.status[1] = 16; prm.status[2] = t0; prm.status[3] = 0;
         }
@@ -419,7 +520,9 @@ decode_kernel(const DecodeParams prm) {
                 z += red[w][r][D + 1] * wgt;
             }
         }
-        const int64_t row = (static_cast<int64_t>(b) * prm.Hq + hk * R + r) * prm.n_splits + split;
+        // partial result of this CTA: balanced, number blockIdx.x of its query head's pool; else [sequence, head, split]
+        const int64_t row = prm.balanced ? static_cast<int64_t>(hk * R + r) * prm.n_ctas + blockIdx.x
+                                         : (static_cast<int64_t>(b) * prm.Hq + hk * R + r) * prm.n_splits + split;
         prm.o_part[row * D + e] = o;
         if (e == 0) { prm.m_part[row] = m; prm.z_part[row] = z; }
     }
@@ -433,15 +536,28 @@ template <int D>
 __global__ void __launch_bounds__(D)
 decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ m_part,
                     const float* __restrict__ z_part, int n_splits, __half* __restrict__ out,
-                    float* __restrict__ lse) {
-    ptx::griddep_wait();   // (when launched as a programmatic dependent of the step kernel)
+                    float* __restrict__ lse, const int32_t* __restrict__ cache_len, int B, int max_len, int Hq) {
     const int64_t row = blockIdx.x;
+    int64_t first = row * n_splits;      // of the row's partial results
+    if (cache_len != nullptr) {          // balanced warp-level form: n_splits is the size of a query head's pool
+        const Shares sh = share_out<kChunk<D>>(cache_len, B, max_len, n_splits);
+        const int b = static_cast<int>(row) / Hq, hq = static_cast<int>(row) - b * Hq;
+        int n = 0, start = sh.start;
+#pragma unroll
+        for (int k = 0; k < kShareRows; ++k) {
+            if (k < b % sh.K) start += sh.s[k];
+            if (k == b % sh.K) n = sh.s[k];
+        }
+        first = static_cast<int64_t>(hq) * n_splits + __shfl_sync(0xffffffffu, start, b / sh.K);
+        n_splits = __shfl_sync(0xffffffffu, n, b / sh.K);
+    }
+    ptx::griddep_wait();   // (when launched as a programmatic dependent of the step kernel)
     const int e = threadIdx.x, lane = e & 31;
     float m = -INFINITY, z = 0.f, o = 0.f;
     for (int s0 = 0; s0 < n_splits; s0 += 32) {
         const int s = s0 + lane;
-        const float ms = s < n_splits ? m_part[row * n_splits + s] : -INFINITY;
-        const float zs = s < n_splits ? z_part[row * n_splits + s] : 0.f;
+        const float ms = s < n_splits ? m_part[first + s] : -INFINITY;
+        const float zs = s < n_splits ? z_part[first + s] : 0.f;
         float mc = ms;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, d));
@@ -452,7 +568,7 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
         const float zw = ms == -INFINITY ? 0.f : zs * w;
         z *= back; o *= back; m = m_new;
         const int cnt = min(32, n_splits - s0);
-        const float* src = o_part + (row * n_splits + s0) * D + e;
+        const float* src = o_part + (first + s0) * D + e;
 #pragma unroll 8
         for (int i = 0; i < cnt; ++i) {
             const float wi = __shfl_sync(0xffffffffu, w, i);
@@ -464,31 +580,49 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
     if (e == 0 && lse != nullptr) lse[row] = z > 0.f ? (m + log2f(z)) * kLn2 : -INFINITY;
 }
 
-template <int D, int R, int T>
-int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t stream) {
-    const dim3 grid(prm.n_splits, prm.Hk, prm.B);
-    constexpr int kRing = kStages * Stage<D, T>::kBytes;   // = kStagesInt8 stages of INT8 keys and values
-    static_assert(kRing == kStagesInt8 * 2 * Stage<D, T>::kV, "both ring shapes fill the same bytes");
-    // no FP16 key cache: the instance whose ring holds three INT8-only stages
-    auto kernel = prm.k16 != nullptr ? decode_kernel<D, R, T, true> : decode_kernel<D, R, T, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRing);
-    if (e != cudaSuccess) return static_cast<int>(e);
-    kernel<<<grid, kDecodeThreads, kRing, stream>>>(prm);
+// Step and merge overlap the tail of the kernel before them (programmatic dependent launch).
+template <int D>
+int launch_merge(const DecodeParams& prm, int n_splits, bool shared, __half* out, float* lse, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(prm.B * prm.Hq); cfg.blockDim = dim3(D); cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_merge_kernel<D>, static_cast<const float*>(prm.o_part),
+                                             static_cast<const float*>(prm.m_part), static_cast<const float*>(prm.z_part),
+                                             n_splits, out, lse, shared ? prm.cache_len_raw : static_cast<const int32_t*>(nullptr),
+                                             prm.B, prm.max_len, prm.Hq);
     g_launch_count.fetch_add(1);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return static_cast<int>(e);
-    decode_merge_kernel<D><<<prm.B * prm.Hq, D, 0, stream>>>(prm.o_part, prm.m_part, prm.z_part, prm.n_splits, out, lse);
-    g_launch_count.fetch_add(1);
-    return static_cast<int>(cudaGetLastError());
+    return static_cast<int>(e);
 }
 
-template <int D, int T>
+template <int D, int R, int RT>
+int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t stream) {
+    // no FP16 key cache: the instance whose ring holds INT8 keys only
+    auto kernel = prm.k16 != nullptr ? decode_kernel<D, R, RT, true> : decode_kernel<D, R, RT, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if (e != cudaSuccess) return static_cast<int>(e);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = prm.balanced ? dim3(prm.n_ctas, prm.Hk) : dim3(prm.n_splits, prm.Hk, prm.B);
+    cfg.blockDim = dim3(kDecodeThreads); cfg.dynamicSmemBytes = kRingBytes; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kernel, prm);
+    g_launch_count.fetch_add(1);
+    if (e != cudaSuccess) return static_cast<int>(e);
+    return launch_merge<D>(prm, prm.balanced ? prm.n_ctas : prm.n_splits, prm.balanced != 0, out, lse, stream);
+}
+
+template <int D, int RT>
 int launch_r(int R, const DecodeParams& prm, __half* out, float* lse, cudaStream_t stream) {
     switch (R) {
-        case 1: return launch_cfg<D, 1, T>(prm, out, lse, stream);
-        case 2: return launch_cfg<D, 2, T>(prm, out, lse, stream);
-        case 4: return launch_cfg<D, 4, T>(prm, out, lse, stream);
-        case 8: return launch_cfg<D, 8, T>(prm, out, lse, stream);
+        case 1: return launch_cfg<D, 1, RT>(prm, out, lse, stream);
+        case 2: return launch_cfg<D, 2, RT>(prm, out, lse, stream);
+        case 4: return launch_cfg<D, 4, RT>(prm, out, lse, stream);
+        case 8: return launch_cfg<D, 8, RT>(prm, out, lse, stream);
         default: return TILEMIX_ERR_UNSUPPORTED;
     }
 }
@@ -553,7 +687,10 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
             if (balance && n_rows <= kDecodeWave && n_rows <= kDecodeBalanceRows) {
                 int row_cap = 8 * splits < 16 ? 16 : 8 * splits;
                 if (row_cap > cap) row_cap = cap;
-                const int64_t ctas = n_rows * row_cap < kDecodeWave ? n_rows * row_cap : kDecodeWave;
+                // With more rows than half a wave a single wave cannot split the long ones: two waves then.
+                // (16 x 8 rows, lengths uniform in [0, 12K]: 82.7 us in one wave, 76.5 in two; the warp-level form 85.)
+                const int64_t most = 2 * n_rows > kDecodeWave ? 2 * kDecodeWave : kDecodeWave;
+                const int64_t ctas = n_rows * row_cap < most ? n_rows * row_cap : most;
                 g->balanced = 1; g->n_ctas = static_cast<int>(ctas); g->split_cap = row_cap;
             }
         } else {
@@ -564,6 +701,16 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
             splits = static_cast<int>(want < 1 ? 1 : want);
             const int cap = g->n_blk / 2 > 0 ? g->n_blk / 2 : 1;
             if (splits > cap) splits = cap;
+            // No more partial results than that, but shared out over the sequences by their cache lengths: one wave of
+            // two CTAs per SM where that is at least two per sequence, else two.  (16 x 8 rows of up to 8K keys, d = 64:
+            // 42 us; with two waves, whose CTAs are shorter and start one behind the other, 48.)
+            if (p->batch <= kMaxShared) {
+                const int64_t wave = 2 * kDecodeWave / p->heads_kv;
+                int64_t pool = p->batch * 2 <= wave ? wave : 2 * wave;
+                if (pool > static_cast<int64_t>(p->batch) * splits) pool = static_cast<int64_t>(p->batch) * splits;
+                if (pool < p->batch) pool = p->batch;
+                g->balanced = 1; g->n_ctas = static_cast<int>(pool);
+            }
         }
     }
     if (splits > g->n_blk) splits = g->n_blk;
@@ -640,20 +787,10 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
         // the tcgen05 form of the step (decode_umma.cu), then the same merge
         rc = launch_decode_umma(R, prm, s);
         if (rc) return rc;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(prm.B * prm.Hq); cfg.blockDim = dim3(128); cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        const cudaError_t me = cudaLaunchKernelEx(&cfg, decode_merge_kernel<128>, static_cast<const float*>(prm.o_part),
-                                                  static_cast<const float*>(prm.m_part), static_cast<const float*>(prm.z_part),
-                                                  g.n_parts, out, lse);
-        g_launch_count.fetch_add(1);
-        return static_cast<int>(me);
+        return launch_merge<128>(prm, g.n_parts, false, out, lse, s);
     }
     if (p->head_dim == 128 && p->tile_n == 64) return launch_r<128, 64>(R, prm, out, lse, s);
-    if (p->head_dim == 64 && p->tile_n == 128) return launch_r<64, kChunk>(R, prm, out, lse, s);
+    if (p->head_dim == 64 && p->tile_n == 128) return launch_r<64, 128>(R, prm, out, lse, s);
     if (p->head_dim == 64 && p->tile_n == 64) return launch_r<64, 64>(R, prm, out, lse, s);
     return TILEMIX_ERR_UNSUPPORTED;
 }
