@@ -1146,11 +1146,15 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapFloatOOBfill);
 
 int get_encoder(EncodeTiledFn* fn) {
-    void* sym = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres);
-    if (e != cudaSuccess) return static_cast<int>(e);
-    if (qres != cudaDriverEntryPointSuccess || sym == nullptr) return static_cast<int>(cudaErrorNotSupported);
+    static std::atomic<void*> encoder{nullptr};      // the driver's tensor-map encoder, looked up once
+    void* sym = encoder.load(std::memory_order_acquire);
+    if (sym == nullptr) {
+        cudaDriverEntryPointQueryResult qres;
+        const cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres);
+        if (e != cudaSuccess) return static_cast<int>(e);
+        if (qres != cudaDriverEntryPointSuccess || sym == nullptr) return static_cast<int>(cudaErrorNotSupported);
+        encoder.store(sym, std::memory_order_release);
+    }
     *fn = reinterpret_cast<EncodeTiledFn>(sym);
     return 0;
 }
@@ -1247,8 +1251,6 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     } else {
         if (prm.k_half_blocks) kernel = pick(std::true_type{});
     }
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
-    if (e != cudaSuccess) return static_cast<int>(e);
     constexpr int kRowsPerCta = 2 * T / C::kRT;          // routing rows of a CTA
     int64_t ctas = vl ? static_cast<int64_t>(g.Hq) * total_pairs
                       : static_cast<int64_t>(g.B) * g.Hq * ceil_div(g.T_m, kRowsPerCta);
@@ -1259,12 +1261,24 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     prm.solo = 2 * ctas <= kSms ? 1 : 0;
     if (prm.solo) ctas *= 2;
     if (ctas > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
-    // The register split inside the kernel (setmaxnreg) assumes what the block is launched with; a build that
-    // gave the kernel fewer registers must not run (an increase beyond the block's allotment never returns).
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kernel);
-    if (e != cudaSuccess) return static_cast<int>(e);
-    if (fa.numRegs < (otf ? kLaunchRegsOtf : kLaunchRegs)) return TILEMIX_ERR_UNSUPPORTED;
+    // Once per device and kernel instance: the shared-memory attribute, and a look at the registers.  The register split
+    // inside the kernel (setmaxnreg) assumes what the block is launched with; a build that gave the kernel fewer registers
+    // must not run (an increase beyond the block's allotment never returns).
+    constexpr int kMaxDev = 64;
+    static std::atomic<uint32_t> prepared[kMaxDev];      // bit per instance
+    const uint32_t bit = 1u << ((vl ? 1 : 0) + (dbg_on ? 2 : 0) + (otf ? 4 : 0) + (v_scale ? 8 : 0) + (prm.k_half_blocks ? 16 : 0));
+    int device = 0;
+    if ((e = cudaGetDevice(&device)) != cudaSuccess) return static_cast<int>(e);
+    const bool known = device >= 0 && device < kMaxDev;
+    if (!known || !(prepared[device].load(std::memory_order_acquire) & bit)) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
+        if (e != cudaSuccess) return static_cast<int>(e);
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, kernel);
+        if (e != cudaSuccess) return static_cast<int>(e);
+        if (fa.numRegs < (otf ? kLaunchRegsOtf : kLaunchRegs)) return TILEMIX_ERR_UNSUPPORTED;
+        if (known) prepared[device].fetch_or(bit, std::memory_order_release);
+    }
     kernel<<<static_cast<unsigned>(ctas), otf ? kThreadsOtf : kThreads, C::kSmemAlloc, stream>>>(prm, tq, tk, tv, tq8, tk8);
     g_launch_count.fetch_add(1);
     return static_cast<int>(cudaGetLastError());

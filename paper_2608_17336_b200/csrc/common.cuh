@@ -49,6 +49,7 @@ struct VarlenTable {
     // four arrays of n + 1 entries (tok, tile, blkq, blkk), then two of total_pairs entries: the
     // attention kernel's work items (sequence, pair of query tiles), longest first
     std::vector<int32_t> tab;
+    size_t used = 0;           // entries that have been filled in: all, or those before the work items
 };
 struct VarlenDev {
     const int32_t* tok = nullptr;    // first token of sequence s (cu_seqlens)
@@ -62,9 +63,9 @@ struct VarlenDev {
 constexpr size_t kStatusAreaBytes = 4096;   // status record, timers, trace: start of every workspace
 
 // Fills `g` for the packed batch (B = 1, L = total tokens, T_m = sum of tile rows, T_mask / W of the
-// longest sequence, T_n = key tiles of the longest sequence) and the prefix sums.
-int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geometry* g, VarlenTable* t);
-// Copies the tables behind the status area of `workspace` on `stream` and points `dev` at them.
+// longest sequence, T_n = key tiles of the longest sequence) and the prefix sums; the work items only if asked for.
+int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geometry* g, VarlenTable* t, bool with_items);
+// Copies the tables (what is filled in of them) behind the status area of `workspace` on `stream` and points `dev` at them.
 int upload_varlen(const VarlenTable& t, void* workspace, cudaStream_t stream, VarlenDev* dev);
 
 #ifdef __CUDACC__

@@ -19,7 +19,7 @@ size_t table_bytes(const VarlenTable& t) { return align_up(t.tab.size() * sizeof
 
 }  // namespace
 
-int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geometry* g, VarlenTable* t) {
+int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geometry* g, VarlenTable* t, bool with_items) {
     if (p == nullptr || vl == nullptr || vl->cu_seqlens == nullptr) return TILEMIX_ERR_NULL;
     if (vl->n_seqs <= 0 || vl->max_seqlen < 0) return TILEMIX_ERR_SHAPE;
     if (p->batch != 1 || p->mask_batch != 1) return TILEMIX_ERR_SHAPE;
@@ -69,19 +69,26 @@ int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geome
     t->total_blk_q = blkq[n];
     t->total_blk_k = blkk[n];
     // Work items of the attention kernel, the longest rows of the whole batch first (a pair p of a
-    // sequence streams 2p + 2 tiles of 128 keys); ties keep the sequence order.
-    std::vector<std::pair<int32_t, int32_t>> items;   // (pair index, sequence)
-    items.reserve(static_cast<size_t>(t->total_pairs));
-    for (int s = 0; s < n; ++s)
-        for (int32_t pr = pair[s + 1] - pair[s] - 1; pr >= 0; --pr) items.emplace_back(pr, s);
-    std::stable_sort(items.begin(), items.end(),
-                     [](const std::pair<int32_t, int32_t>& a, const std::pair<int32_t, int32_t>& b) { return a.first > b.first; });
-    const size_t base = t->tab.size();
-    t->tab.resize(base + 2u * items.size());
-    for (size_t i = 0; i < items.size(); ++i) {
-        t->tab[base + i] = items[i].second;
-        t->tab[base + items.size() + i] = items[i].first;
+    // sequence streams 2p + 2 tiles of 128 keys); equal ones in sequence order.
+    const size_t base = t->tab.size(), n_items = static_cast<size_t>(t->total_pairs);
+    t->tab.resize(base + 2u * n_items);
+    if (with_items) {
+        int32_t longest_pair = 0;
+        for (int s = 0; s < n; ++s) longest_pair = std::max(longest_pair, pair[s + 1] - pair[s]);
+        // first place of the items with pair index p: behind those with a larger one (counted, not sorted)
+        std::vector<int32_t> place(static_cast<size_t>(longest_pair) + 1u, 0);
+        for (int s = 0; s < n; ++s)
+            for (int32_t p_ = pair[s + 1] - pair[s] - 1; p_ >= 0; --p_) ++place[static_cast<size_t>(p_)];
+        int32_t at = 0;
+        for (int32_t p_ = longest_pair - 1; p_ >= 0; --p_) { const int32_t c = place[static_cast<size_t>(p_)]; place[static_cast<size_t>(p_)] = at; at += c; }
+        for (int s = 0; s < n; ++s)
+            for (int32_t p_ = 0; p_ < pair[s + 1] - pair[s]; ++p_) {
+                const size_t i = static_cast<size_t>(place[static_cast<size_t>(p_)]++);
+                t->tab[base + i] = s;
+                t->tab[base + n_items + i] = p_;
+            }
     }
+    t->used = with_items ? t->tab.size() : base;
     g->T_m = t->total_tiles;
     g->mask_T_m = t->total_tiles;
     g->T_n = static_cast<int>(ceil_div(t->max_len, g->tile_n));
@@ -93,7 +100,7 @@ int resolve_varlen(const tilemix_problem_t* p, const tilemix_varlen_t* vl, Geome
 int upload_varlen(const VarlenTable& t, void* workspace, cudaStream_t stream, VarlenDev* dev) {
     int32_t* base = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + kStatusAreaBytes);
     // The source is pageable host memory: the runtime has staged it by the time the call returns.
-    const cudaError_t e = cudaMemcpyAsync(base, t.tab.data(), t.tab.size() * sizeof(int32_t),
+    const cudaError_t e = cudaMemcpyAsync(base, t.tab.data(), t.used * sizeof(int32_t),
                                           cudaMemcpyHostToDevice, stream);
     if (e != cudaSuccess) return static_cast<int>(e);
     const int n1 = t.n + 1;
@@ -114,7 +121,7 @@ int tilemix_varlen_counts(const tilemix_problem_t* p, const tilemix_varlen_t* vl
     if (out == nullptr) return TILEMIX_ERR_NULL;
     Geometry g;
     VarlenTable t;
-    const int rc = resolve_varlen(p, vl, &g, &t);
+    const int rc = resolve_varlen(p, vl, &g, &t, false);
     if (rc) return rc;
     out[0] = g.L; out[1] = t.total_tiles; out[2] = t.total_blk_q; out[3] = t.total_blk_k;
     out[4] = g.T_mask; out[5] = g.W; out[6] = t.max_len;
@@ -124,7 +131,7 @@ int tilemix_varlen_counts(const tilemix_problem_t* p, const tilemix_varlen_t* vl
 size_t tilemix_varlen_workspace_size(const tilemix_problem_t* p, const tilemix_varlen_t* vl) {
     Geometry g;
     VarlenTable t;
-    if (resolve_varlen(p, vl, &g, &t)) return 0;
+    if (resolve_varlen(p, vl, &g, &t, false)) return 0;
     return kStatusAreaBytes + table_bytes(t);
 }
 
@@ -133,7 +140,7 @@ int tilemix_quantize_qk_varlen(const tilemix_problem_t* p, const tilemix_varlen_
                                void* workspace, size_t workspace_bytes, void* stream) {
     Geometry g;
     VarlenTable t;
-    int rc = resolve_varlen(p, vl, &g, &t);
+    int rc = resolve_varlen(p, vl, &g, &t, false);
     if (rc) return rc;
     const bool do_q = q_f16 || q_i8 || q_scale, do_k = k_f16 || k_i8 || k_scale;
     if ((!do_q && !do_k) || workspace == nullptr) return TILEMIX_ERR_NULL;
@@ -163,7 +170,7 @@ int tilemix_pack_routing_mask_varlen(const tilemix_problem_t* p, const tilemix_v
                                      size_t workspace_bytes, void* stream) {
     Geometry g;
     VarlenTable t;
-    int rc = resolve_varlen(p, vl, &g, &t);
+    int rc = resolve_varlen(p, vl, &g, &t, false);
     if (rc) return rc;
     if (route == nullptr || mask_words == nullptr || workspace == nullptr) return TILEMIX_ERR_NULL;
     if (!aligned16(workspace)) return TILEMIX_ERR_ALIGN;
@@ -181,7 +188,7 @@ int tilemix_attention_fwd_varlen(const tilemix_problem_t* p, const tilemix_varle
                                  const tilemix_debug_t* dbg, void* stream) {
     Geometry g;
     VarlenTable t;
-    int rc = resolve_varlen(p, vl, &g, &t);
+    int rc = resolve_varlen(p, vl, &g, &t, true);
     if (rc) return rc;
     if (!q_f16 || !k_f16 || !v_f16 || !out_f16 || !workspace) return TILEMIX_ERR_NULL;
     if ((g.flags & TILEMIX_QUANT_ON_THE_FLY) != 0) return TILEMIX_ERR_UNSUPPORTED;   // dense batches only
