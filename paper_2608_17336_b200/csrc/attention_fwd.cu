@@ -1,8 +1,9 @@
 // Fused TileMix attention forward for sm_100a (Sec. 4.1 loops, Sec. 4.3 "Tile-group dispatch",
 // Sec. 3.1 online softmax, App. C score formulas).
 //
-// One CTA owns two adjacent query tiles (A = 2p, B = 2p+1) of one (batch, query head) and
-// streams the key/value tiles 0..B once for both.  Warp roles (w = warp index):
+// One CTA owns two query tiles A and B -- two adjacent ones of one (batch, query head), or the same rows of two query
+// heads that share a KV head -- and streams the key/value tiles up to their diagonal once for both.  Warp roles (w =
+// warp index):
 //   warps 0-15  softmax warps: tile (w >> 2) & 1, 16 query rows each -- TMEM lanes 32 (w & 3) + 16 (w >> 3)
 //               .. + 15 (a warp may only touch the lane quarter w & 3), read in the 16-lane shapes so that the
 //               four warps of a scheduler work on four disjoint sets of rows
@@ -11,7 +12,7 @@
 //   warps 17,18 MMA issuers, one per query tile: tcgen05.mma kind::f16 or kind::i8 for S = Q K^T per the
 //               routing bit, then kind::f16 for O += P V with P read from tensor memory; warp 17 also owns
 //               the TMEM allocation.  The whole warp runs the loop, one elected lane issues.
-//   warp  19    idle
+//   warp  19    scale warp: the factors the softmax warps multiply their accumulators with (not in the on-the-fly mode)
 //   warps 20-23 only in the on-the-fly operand mode: the on-chip quantiser, which makes the INT8 copies of
 //               the query tiles and of the key tiles routed to INT8 in shared memory from the FP16 tiles
 // Tensor memory: S_A | S_B | O_A | O_B (FP32 / INT32 accumulators).  A score tile is produced and consumed in
@@ -131,7 +132,7 @@ struct Params {
     int test_drop_bundle;              // testing aid: the producer leaves out the copies of this operand bundle (-1: none)
     int head_group;               // (batch, head) rows interleaved in the grid order (>= 1)
     int has_int8;                 // INT8 operands present
-    int solo;                     // 1: one tile per CTA (small grids), 0: two
+    int single;                   // 1: a CTA has one row of tiles (of one head, or of two), 0: two adjacent ones of one head
     float scale_log2;             // softmax scale * log2(e)
     const float* q_scale;         // [B,Hq,T_m]; variable-length batch: [sum T_m, Hq]
     const float* k_scale;         // [B,Hk,T_n]; variable-length batch: [sum T_n, Hk]
@@ -213,7 +214,9 @@ struct Ring {
 // of the other instances is ~1 % faster without that code in it.
 // KH (head dimension 64): quantisation blocks of K of half a routing tile, i.e. two scales per step.  (Head dimension
 // 128 has one scale per step either way and takes both at run time.)
-template <int D, bool VL, bool OTF, bool VS = false, bool DBG = false, bool KH = false>
+// HP: tiles A and B are the same rows of two query heads of one KV head (an instance of its own: the index arithmetic of
+// both cost the other form 0.5-0.8 %).
+template <int D, bool VL, bool OTF, bool VS = false, bool DBG = false, bool KH = false, bool HP = false>
 __global__ void __launch_bounds__(OTF ? kThreadsOtf : kThreads, 1)
 attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                  const __grid_constant__ CUtensorMap tm_k16, const __grid_constant__ CUtensorMap tm_v16,
@@ -243,27 +246,29 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     // first, and the heads of the group side by side for each item.  The host sizes the group so that its
     // K/V fits in L2 while its CTAs run; the grid then ends with the shortest items of the last group instead
     // of with the long items of the last head, and the SMs finish close together.
-    // With `solo` two adjacent CTAs take the two tiles of a pair (the longer one first).
+    // With `single` two adjacent CTAs take the two tiles of a pair (the longer one first).
     const int kHeadGroup = prm.head_group;
-    const int blk = static_cast<int>(blockIdx.x) >> prm.solo;
+    const int blk = static_cast<int>(blockIdx.x) >> prm.single;
+    constexpr int hp = HP ? 1 : 0;
+    const int n_heads = prm.Hq >> hp;   // (heads, or pairs of heads)
     if constexpr (!VL) {
         const int n_pairs = SUB ? (prm.T_m + 3) >> 2 : (prm.T_m + 1) >> 1;
-        const int n_bh = prm.B * prm.Hq;
+        const int n_bh = prm.B * n_heads;
         const int grp = blk / (kHeadGroup * n_pairs);
         const int in_grp = blk - grp * (kHeadGroup * n_pairs);
         const int g_heads = min(kHeadGroup, n_bh - grp * kHeadGroup);    // the last group may be smaller
         const int item = in_grp / g_heads;
         const int bh = grp * kHeadGroup + (in_grp - item * g_heads);
         pr = n_pairs - 1 - item;                            // longest rows first
-        b = bh / prm.Hq;
-        hq = bh - b * prm.Hq;
+        b = bh / n_heads;
+        hq = (bh - b * n_heads) << hp;
         seq = b;
     } else {
         const int grp = blk / (kHeadGroup * prm.total_pairs);
         const int in_grp = blk - grp * (kHeadGroup * prm.total_pairs);
-        const int g_heads = min(kHeadGroup, prm.Hq - grp * kHeadGroup);
+        const int g_heads = min(kHeadGroup, n_heads - grp * kHeadGroup);
         const int item = in_grp / g_heads;                  // items are sorted by length on the host
-        hq = grp * kHeadGroup + (in_grp - item * g_heads);
+        hq = (grp * kHeadGroup + (in_grp - item * g_heads)) << hp;
         seq = prm.vl_item_seq[item];
         pr = prm.vl_item_pair[item];
         b = 0;
@@ -281,10 +286,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     // not exist, and a chunk may begin in the middle of a key tile, so that number may be odd).
     const int kv_off = VL ? 0 : prm.kv_off;
     const int n_tiles = SUB ? (n_rows + 1) >> 1 : n_rows;
-    const int mA = prm.solo ? 2 * pr + 1 - static_cast<int>(blockIdx.x & 1) : 2 * pr, mB = mA + 1;
-    if (prm.solo && mA >= n_tiles) return;
-    const bool hasB = !prm.solo && mB < n_tiles;
-    const int dA = SUB ? kv_off + 2 * mA : 2 * (mA + kv_off), dB = dA + 2;
+    const int mA = prm.single ? 2 * pr + 1 - static_cast<int>(blockIdx.x & 1) : 2 * pr, mB = hp ? mA : mA + 1;
+    if (prm.single && mA >= n_tiles) return;
+    const bool hasB = hp || (!prm.single && mB < n_tiles);
+    const int dA = SUB ? kv_off + 2 * mA : 2 * (mA + kv_off), dB = SUB ? kv_off + 2 * mB : 2 * (mB + kv_off);
     const int uA = SUB ? kv_off + min(2 * mA + 2, n_rows) : dA + 2;
     const int uB = SUB ? kv_off + min(2 * mB + 2, n_rows) : dB + 2;
     const int nkv = ((hasB ? uB : uA) + 1) >> 1;
@@ -369,9 +374,9 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 ptx::mbar_arrive_expect_tx(bar_q(t), bytes);
                 for (int c = 0; c < C::kHalves; ++c)
                     ptx::tma_load_4d(sbase + C::kOffQ16 + t * C::kQ16Tile + c * C::kQ16Slab, &tm_q16,
-                                     bar_q(t), c * 64, tok0 + m * T, hq, b);
+                                     bar_q(t), c * 64, tok0 + m * T, hq + (t ? hp : 0), b);
                 if (prm.has_int8 && !OTF)
-                    ptx::tma_load_4d(sbase + C::kOffQ8 + t * C::kQ8Tile, &tm_q8, bar_q(t), 0, tok0 + m * T, hq, b);
+                    ptx::tma_load_4d(sbase + C::kOffQ8 + t * C::kQ8Tile, &tm_q8, bar_q(t), 0, tok0 + m * T, hq + (t ? hp : 0), b);
             }
             if (!OTF) {
                 ptx::mbar_arrive_expect_tx(bar_full(0), C::kHalves * C::kChunk + (prm.has_int8 ? C::kK8Bytes : 0));
@@ -394,7 +399,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         const int j0 = i * 8, j_last = min(j0 + 7, n_entries - 1);
         constexpr int NR = SUB ? 4 : 2;                // routing rows of this CTA: mrow .. mrow + NR - 1
         const int mrow = SUB ? 2 * mA : mA;
-        const int n_live = min(hasB ? NR : NR / 2, n_rows - mrow);
+        const int n_live = min(hasB && !hp ? NR : NR / 2, n_rows - mrow);
         int g = 0, in_g = 0, w_lo = 0;
         uint32_t wr[NR][2];
 #pragma unroll
@@ -431,8 +436,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         else if (r >= n_live) e = (e & ~(1u << r)) | (last << r);
                     }
                 }
+                if (hp) e = (e & 3u) * 5u;                     // tile B has tile A's rows
                 before = e;
             } else {
+                if (hp) e = (e & 1u) * 3u;
                 const bool useA = j <= mA + kv_off;
                 if ((useA && !(e & 1u)) || (hasB && !(e & 2u))) e |= 4u;
                 if ((useA && (e & 1u)) || (hasB && (e & 2u))) e |= 8u;
@@ -608,8 +615,9 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         const bool mine = lane < kNumSc && prm.has_int8;
         // scales: dense [B,H,blocks] (unit stride over blocks), variable-length [blocks, H]
         float dq = 0.f;
-        if (mine) dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + row) * prm.Hq + hq]
-                              : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.T_m + row];
+        const int hq_t = hq + (t ? hp : 0);
+        if (mine) dq = varlen ? prm.q_scale[static_cast<int64_t>(row0 + row) * prm.Hq + hq_t]
+                              : prm.q_scale[(static_cast<int64_t>(b) * prm.Hq + hq_t) * prm.T_m + row];
         const float* dk_row = varlen ? prm.k_scale + static_cast<int64_t>(kblk0) * prm.Hk + hk
                                      : prm.k_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.ks_blocks;
         const float* dv_row = VS ? prm.v_scale + (static_cast<int64_t>(b) * prm.Hk + hk) * prm.vs_blocks : nullptr;
@@ -1010,7 +1018,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         if (lane == 0) {
                             for (int e = 0; e < prm.dbg_n; ++e) {
                                 const int32_t* qd = prm.dbg_tiles + 4 * e;
-                                if (qd[0] == seq && qd[1] == hq && qd[2] == (SUB ? 2 * m_t + rh : m_t) && qd[3] == (SUB ? u : j)) { idx = e; break; }
+                                if (qd[0] == seq && qd[1] == hq + (t ? hp : 0) && qd[2] == (SUB ? 2 * m_t + rh : m_t) && qd[3] == (SUB ? u : j)) { idx = e; break; }
                             }
                         }
                         idx = __shfl_sync(0xffffffffu, idx, 0);
@@ -1128,12 +1136,12 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     const bool row_valid = i_loc < len;
                     z[k] = row_valid ? 1.f / z_row : 0.f;
                     if (row_valid && cq == 0 && prm.lse != nullptr)
-                        prm.lse[(static_cast<int64_t>(b) * prm.Hq + hq) * prm.L + i_glob] = (m_run[k] + log2f(z_row)) * kLn2;
+                        prm.lse[(static_cast<int64_t>(b) * prm.Hq + hq + (t ? hp : 0)) * prm.L + i_glob] = (m_run[k] + log2f(z_row)) * kLn2;
                 }
                 // Two adjacent columns per lane and block of 8: a 4 x 4 transpose inside the quad gives every lane one
                 // whole block, so that a row leaves in 16-byte pieces; 4-byte stores touch every line four times as often.
                 // (8 x 4K: 1193 -> 1181 us; packed batch of 16 prompts: 515 -> 506)
-                __half* dst0 = prm.out + b * prm.os[0] + hq * prm.os[1] + (static_cast<int64_t>(tok0) + m_t * T) * prm.os[2] + 8 * (lane & 3);
+                __half* dst0 = prm.out + b * prm.os[0] + (hq + (t ? hp : 0)) * prm.os[1] + (static_cast<int64_t>(tok0) + m_t * T) * prm.os[2] + 8 * (lane & 3);
                 const bool odd = lane & 1, upper = lane & 2;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
@@ -1243,15 +1251,6 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     prm.k_half_blocks = (g.blk_k * 2 == g.tile_n) ? 1 : 0;
     prm.wait_limit_ns = g_wait_limit_ns.load();
     prm.test_drop_bundle = g_test_drop.load() == 1 ? 1 : -1;
-    {
-        // heads per group: as many as keep the group's K and V (FP16; adjacent query heads of a GQA group share
-        // theirs) within 72 MB of the 126 MB L2
-        const int64_t kv_bytes = 2 * static_cast<int64_t>(g.Lk) * g.d * 2;
-        const int rep = g.Hq / g.Hk;
-        int hg = 1;
-        while (hg < kMaxHeadGroup && ceil_div(2 * hg, rep) * kv_bytes <= (72ll << 20)) hg *= 2;
-        prm.head_group = hg;
-    }
     prm.nb = g.nb;
     prm.has_int8 = has8 ? 1 : 0;
     prm.scale_log2 = g.scale * kLog2e;
@@ -1273,18 +1272,6 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     if (e != cudaSuccess) return static_cast<int>(e);
     const bool dbg_on = prm.dbg_n > 0;
     if (v_scale != nullptr && dbg_on) return TILEMIX_ERR_UNSUPPORTED;     // (the chunk against an INT8 value cache has no debug instance)
-    auto pick = [&](auto kh) {
-        constexpr bool KH = decltype(kh)::value;
-        if (v_scale != nullptr) return attention_kernel<D, false, false, true, false, KH>;
-        return vl ? (dbg_on ? attention_kernel<D, true, false, false, true, KH> : attention_kernel<D, true, false, false, false, KH>)
-                  : (dbg_on ? attention_kernel<D, false, false, false, true, KH> : attention_kernel<D, false, false, false, false, KH>);
-    };
-    auto kernel = pick(std::false_type{});
-    if constexpr (D == 128) {
-        if (otf) kernel = dbg_on ? attention_kernel<D, false, true, false, true> : attention_kernel<D, false, true>;
-    } else {
-        if (prm.k_half_blocks) kernel = pick(std::true_type{});
-    }
     constexpr int kRowsPerCta = 2 * T / C::kRT;          // routing rows of a CTA
     int64_t ctas = vl ? static_cast<int64_t>(g.Hq) * total_pairs
                       : static_cast<int64_t>(g.B) * g.Hq * ceil_div(g.T_m, kRowsPerCta);
@@ -1292,15 +1279,52 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
     // A grid that leaves half of the SMs idle gives every tile a CTA (and special-function units) of its own: 8 heads x
     // 1000 tokens, d = 128, whole step 42 -> 36 us; 4 x 2000 60 -> 50; 1 x 4096 87 -> 73; 4 x 1000, d = 64 40 -> 36.
     // Beyond that line pairs win: they read every key tile once for two query tiles and still fit one wave.
-    prm.solo = 2 * ctas <= kSms ? 1 : 0;
-    if (prm.solo) ctas *= 2;
+    const int rep = g.Hq / g.Hk;
+    bool head_pair = false;
+    if (2 * ctas <= kSms) {
+        prm.single = 1;
+        ctas *= 2;
+    } else if (rep % 2 == 0 && !dbg_on) {
+        // Query heads that share a KV head share its routing rows and their diagonal.  Tiles A and B of a CTA are then the
+        // same rows of two such heads: both take the same form of every key tile (adjacent rows of one head differ in 37 %
+        // of the tiles at 75 % INT8, and then both copies have to be brought, 80 of the ring's 128 KB) and neither waits
+        // for the other's last tile.  32 / 8 heads: 2048-token chunk of 24K 705 -> 645 us, packed batch of 16 prompts
+        // 515 -> 483, 8K 474 -> 450, the same on the fly 661 -> 633, 4 x 2K without INT8 groups 208 -> 202, 8 x 500 equal;
+        // 28 / 14 heads, 2 x 3000, 90 % INT8: 173 -> 175.
+        head_pair = true;
+        prm.single = 1;                            // (half as many pairs of heads, two CTAs per pair of tiles)
+    }
+    {
+        // heads (pairs of heads) per group: as many as keep the group's K and V (FP16; the query heads of a GQA group share
+        // theirs) within 72 MB of the 126 MB L2
+        const int64_t kv_bytes = 2 * static_cast<int64_t>(g.Lk) * g.d * 2;
+        const int per = head_pair ? 2 : 1;
+        int hg = 1;
+        while (hg < kMaxHeadGroup && ceil_div(2 * hg * per, rep) * kv_bytes <= (72ll << 20)) hg *= 2;
+        prm.head_group = hg;
+    }
+    auto pick = [&](auto kh) {
+        constexpr bool KH = decltype(kh)::value;
+        if (head_pair) return v_scale != nullptr ? attention_kernel<D, false, false, true, false, KH, true>
+                              : vl ? attention_kernel<D, true, false, false, false, KH, true> : attention_kernel<D, false, false, false, false, KH, true>;
+        if (v_scale != nullptr) return attention_kernel<D, false, false, true, false, KH>;
+        return vl ? (dbg_on ? attention_kernel<D, true, false, false, true, KH> : attention_kernel<D, true, false, false, false, KH>)
+                  : (dbg_on ? attention_kernel<D, false, false, false, true, KH> : attention_kernel<D, false, false, false, false, KH>);
+    };
+    auto kernel = pick(std::false_type{});
+    if constexpr (D == 128) {
+        if (otf) kernel = dbg_on ? attention_kernel<D, false, true, false, true>
+                                 : head_pair ? attention_kernel<D, false, true, false, false, false, true> : attention_kernel<D, false, true>;
+    } else {
+        if (prm.k_half_blocks) kernel = pick(std::true_type{});
+    }
     if (ctas > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
     // Once per device and kernel instance: the shared-memory attribute, and a look at the registers.  The register split
     // inside the kernel (setmaxnreg) assumes what the block is launched with; a build that gave the kernel fewer registers
     // must not run (an increase beyond the block's allotment never returns).
     constexpr int kMaxDev = 64;
-    static std::atomic<uint32_t> prepared[kMaxDev];      // bit per instance
-    const uint32_t bit = 1u << ((vl ? 1 : 0) + (dbg_on ? 2 : 0) + (otf ? 4 : 0) + (v_scale ? 8 : 0) + (prm.k_half_blocks ? 16 : 0));
+    static std::atomic<uint64_t> prepared[kMaxDev];      // bit per instance
+    const uint64_t bit = 1ull << ((vl ? 1 : 0) + (dbg_on ? 2 : 0) + (otf ? 4 : 0) + (v_scale ? 8 : 0) + (prm.k_half_blocks ? 16 : 0) + (head_pair ? 32 : 0));
     int device = 0;
     if ((e = cudaGetDevice(&device)) != cudaSuccess) return static_cast<int>(e);
     const bool known = device >= 0 && device < kMaxDev;
