@@ -506,8 +506,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         ptx::setmaxnreg_dec<OTF ? kRegsOtherOtf : kRegsOther>();
         static_assert(!OTF || (D == 128 && T == 128), "the on-chip quantiser handles 128 x 128 tiles");
         const int cw = warp - kQuantWarp0;
-        volatile uint32_t* xch = misc + 2;   // partial maxima of the four warps: words 2, 3, 14, 15 of misc
-        auto xch_slot = [&](int w) -> volatile uint32_t& { return xch[w < 2 ? w : w + 10]; };
+        // Partial maxima of the four warps, in two sets of words by the parity of the tile: a set is written again two
+        // tiles later, behind the next tile's barrier, so one barrier per tile is enough.
+        volatile uint32_t* xch = misc + 4;
+        int xset = 0;
         // `ok` turns false when a bounded wait ran out or the CTA is aborting; a warp then skips the work but
         // keeps meeting the others at the named barrier (every warp runs the same number of tiles).
         bool ok = true;
@@ -525,17 +527,17 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         v[u] = *reinterpret_cast<const uint4*>(src + (sl * 1024 + cw * kVecW + lane + 32 * u) * 16);
 #pragma unroll
                     for (int u = 0; u < kVecW / 32; ++u)
-                        amax2 = umax2(amax2, umax2(umax2(habs2_bits(v[u].x), habs2_bits(v[u].y)),
-                                                   umax2(habs2_bits(v[u].z), habs2_bits(v[u].w))));
+                        amax2 = hmaxabs2(hmaxabs2(amax2, hmaxabs2(v[u].x, v[u].y)), hmaxabs2(v[u].z, v[u].w));
                 }
             }
+            amax2 = habs2_bits(amax2);
             uint32_t amax = max(amax2 & 0xffffu, amax2 >> 16);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-            if (lane == 0) xch_slot(cw) = amax;
+            if (lane == 0) xch[xset + cw] = amax;
             ptx::bar_sync_named(kQuantBar, kQuantWarps * 32);
-            amax = max(max(xch_slot(0), xch_slot(1)), max(xch_slot(2), xch_slot(3)));
-            ptx::bar_sync_named(kQuantBar, kQuantWarps * 32);   // all have read: the slots may be written again
+            amax = max(max(xch[xset], xch[xset + 1]), max(xch[xset + 2], xch[xset + 3]));
+            xset ^= 4;
             const float amax_f = __half2float(__ushort_as_half(static_cast<unsigned short>(amax)));
             QuantScale qs = quant_scale(amax_f);
             if (!ok) return qs.delta;

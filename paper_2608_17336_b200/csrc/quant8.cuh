@@ -10,6 +10,14 @@ namespace tilemix {
 
 __device__ __forceinline__ uint32_t habs2_bits(uint32_t v) { return v & 0x7fff7fffu; }
 
+// Larger magnitude of two packed pairs of binary16 values in one instruction; the sign bits of the result mean
+// nothing (habs2_bits when the last one is in).  For the on-chip quantiser, which is bound by its instructions.
+__device__ __forceinline__ uint32_t hmaxabs2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.NaN.xorsign.abs.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // max of two packed pairs of non-negative binary16 values: for non-negative finite halves the
 // bit patterns order like unsigned integers.
 __device__ __forceinline__ uint32_t umax2(uint32_t a, uint32_t b) { return __vmaxu2(a, b); }
