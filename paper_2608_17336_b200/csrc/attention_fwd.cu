@@ -653,7 +653,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             if (!ok) break;
             if (n < nkv) {
                 const uint32_t e = sched(n);
-                const uint32_t r = SUB ? (e >> (4 * h + 2 * t + rh)) & 1u : (e >> t) & 1u;
+                uint32_t r = SUB ? (e >> (4 * h + 2 * t + rh)) & 1u : (e >> t) & 1u;
+                // keys above the diagonal of these rows: all masked, so the factor is one that is finite (delta_K is
+                // not where a key of the block is not)
+                if (SUB && 2 * n + h > (t ? dB : dA) + rh) r = 0u;
                 if (lane < kNumSc + (VS ? 2 : 0))
                     sc_s[(n % C::kScSlots) * C::kScStride + lane] = lane < kNumSc ? factor(r, dq, cur) : cur;
             }
@@ -867,11 +870,19 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 }
             };
             // O_t (+)= P_t V_j over the keys of half h, with P in tensor memory (two FP16 per 32-bit
-            // column, at the start of its own half of S_t)
-            auto issue_pv = [&](int t, int h, uint32_t sv, uint32_t accumulate) {
+            // column, at the start of its own half of S_t).  `above` (D = 64, never the first step): the keys lie above
+            // the diagonal of the first row half.  Its P is 0 there, but 0 times a value that is not finite is not, so
+            // its lanes are switched off: a row sees V of no key beyond its own 64-key tile.
+            auto issue_pv = [&](int t, int h, uint32_t sv, uint32_t accumulate, bool above) {
                 const uint32_t d_tmem = tmem_base + 2 * C::kSCols + t * C::kOCols;
                 const uint32_t a_tmem = tmem_base + t * C::kSCols + h * TH;
                 const uint32_t b_lo = ring_lo_v + sv * kChunkLo + h * (TH / 16) * 128;
+                if (SUB && above) {
+#pragma unroll
+                    for (int k = 0; k < TH / 16; ++k)
+                        ptx::mma_f16_ts_lanes<true>(d_tmem, a_tmem + k * 8, b_lo + k * 128, kHi16, kIdescPV, 0xffffffffu, 0u);
+                    return;
+                }
                 ptx::mma_f16_ts(d_tmem, a_tmem, b_lo, kHi16, kIdescPV, accumulate);
 #pragma unroll
                 for (int k = 1; k < TH / 16; ++k)
@@ -914,7 +925,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         if (SUB && 2 * j + h >= u_t) break;
                         if (!wait_bar(cx, bar_p(t, h), j & 1, kRoleMma, j, kBarP)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
-                        issue_pv(t, h, sv, (j > 0 || h > 0) ? 1u : 0u);
+                        issue_pv(t, h, sv, (j > 0 || h > 0) ? 1u : 0u, SUB && 2 * j + h > (t ? dB : dA));
                         if (2 * j + h == u_t - 2) ptx::mma_commit(bar_pv(t));   // the last-but-one PV (a rescale in the last step waits for it)
                         if (2 * j + h == u_t - 1) ptx::mma_commit(bar_o(t));
                         if (2 * (j + 1) + h < u_t) {
