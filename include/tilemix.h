@@ -302,15 +302,13 @@ typedef struct tilemix_decode {
     int32_t max_len;       /* token capacity of the caches (their token stride)             */
     int32_t tile_n, group; /* key tile = scale block; G key tiles per routing bit           */
     int32_t mask_batch;    /* 1 = one mask row per KV head shared by the batch, or == batch */
-    int32_t n_splits;      /* CTAs per (b, h_k); 0 = chosen by the library: the same for every (b, h_k) in the tcgen05
-                            * form, by the sequences' cache lengths in the warp-level form (batch <= 256; the order
-                            * of a sequence's FP32 sums then depends on the lengths beside it: pass a count > 0 where
-                            * that matters);
+    int32_t n_splits;      /* CTAs per (b, h_k); 0 = chosen by the library, the same for every (b, h_k);
                             * -1 = chosen by the kernel per (b, h_k), for batches of unequal cache lengths: in
                             * the tcgen05 form with batch * heads_kv <= 148 the CTAs of one wave (two, with more than
                             * 74 rows) are shared out so that the largest number of cache bytes a CTA reads is as
                             * small as it can be (a row gets clamp(ceil(bytes / tau), 1, cap) CTAs for the smallest
-                            * tau that fits); elsewhere -1 means 0 */
+                            * tau that fits); elsewhere -1 means 0.  Except in that shared-out form, what a sequence's
+                            * result is does not depend on the lengths beside it. */
     float softmax_scale;   /* <= 0 means 1/sqrt(head_dim)                                   */
 } tilemix_decode_t;
 

@@ -40,57 +40,44 @@ struct Stage {
 };
 constexpr int kMaxStages = 6;
 
-// Rows of unequal cache lengths (the library chooses the splits): the `pool` partial results that a KV head's workspace
-// has room for are shared out over the sequences by their length, s_b = max(1, ceil(tiles_b / q)) CTAs to sequence b for
-// the smallest q whose total fits, so that the CTAs of the grid finish together.  Lane l of a warp works on sequences
-// l * K .. l * K + K - 1 (K = ceil(B / 32) <= kShareRows); every warp that asks finds the same shares.
-constexpr int kShareRows = 8, kMaxShared = 32 * kShareRows;
-struct Shares {
-    int s[kShareRows];   // CTAs of this lane's sequences
-    int start;           // first CTA of the lane's first sequence
-    int K;
-};
+// Sequence number n of the batch (0: the longest) by cache length in kernel tiles, equal ones in their order.  The grid
+// takes the sequences in this order, so that it ends with the shortest CTAs; which keys a CTA gets does not depend on it.
+// (Up to 8K keys each, 32 / 8 heads of 64: 16 sequences of four splits 50 us in the order of the batch, 42 so; 64 of up to
+// 4K keys, one split each, 77 and 65.)
+// Lane l holds the lengths of sequences l, l + 32, ...; a radix selection on (tiles, ~sequence), the same in every warp.
+constexpr int kSortRows = 8, kMaxSorted = 32 * kSortRows;
 template <int T>
-__device__ __forceinline__ Shares share_out(const int32_t* __restrict__ cache_len, int B, int max_len, int pool) {
-    const int lane = threadIdx.x & 31;
-    Shares sh;
-    sh.K = (B + 31) >> 5;
-    int tiles[kShareRows], total = 0, longest = 1;
+__device__ __forceinline__ int nth_longest(const int32_t* __restrict__ cache_len, int B, int max_len, int n) {
+    const int lane = threadIdx.x & 31, index_bits = B <= 32 ? 5 : 8, last = (1 << index_bits) - 1;
+    uint32_t key[kSortRows], most = 0u, least = 0xffffffffu;      // (key 0: no such sequence)
 #pragma unroll
-    for (int k = 0; k < kShareRows; ++k) {
-        const int b = lane * sh.K + k;
-        tiles[k] = k < sh.K && b < B ? (min(max(cache_len[b], 0), max_len) + T - 1) / T : -1;
-        total += max(tiles[k], 0);
-        longest = max(longest, tiles[k]);
+    for (int k = 0; k < kSortRows; ++k) {
+        const int b = lane + 32 * k;
+        key[k] = 0u;
+        if (b < B) {
+            const uint32_t tiles = min((min(max(cache_len[b], 0), max_len) + T - 1) / T, (1 << 23) - 2);
+            key[k] = (tiles + 1) << index_bits | static_cast<uint32_t>(last - b);
+            most = max(most, key[k]);
+            least = min(least, key[k]);
+        }
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    least = __reduce_min_sync(0xffffffffu, least);
+    if (most >> index_bits == least >> index_bits) return n;     // all of one length
+    uint32_t found = 0u;
+    for (int bit = 31 - __clz(most); bit >= 0; --bit) {
+        const uint32_t want = (found >> bit) | 1u;
+        int with_bit = (key[0] >> bit) == want ? 1 : 0;
+        if (index_bits > 5) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        total += __shfl_xor_sync(0xffffffffu, total, o);
-        longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, o));
+            for (int k = 1; k < kSortRows; ++k) with_bit += (key[k] >> bit) == want ? 1 : 0;
+            with_bit = __reduce_add_sync(0xffffffffu, with_bit);
+        } else {
+            with_bit = __popc(__ballot_sync(0xffffffffu, with_bit));
+        }
+        if (n < with_bit) found |= 1u << bit; else n -= with_bit;
     }
-    auto share = [&](int t, int q) -> int { return t < 0 ? 0 : max(1, (t + q - 1) / q); };
-    int lo = max(1, (total + pool - 1) / pool);
-    int hi = pool > B ? max(lo, min(longest, (total + pool - B - 1) / (pool - B))) : max(lo, longest);   // fits: sum of ceil(t / q) <= total / q + B
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        int n = 0;
-#pragma unroll
-        for (int k = 0; k < kShareRows; ++k) n += share(tiles[k], mid);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-        if (n <= pool) hi = mid; else lo = mid + 1;
-    }
-    int mine = 0;
-#pragma unroll
-    for (int k = 0; k < kShareRows; ++k) { sh.s[k] = share(tiles[k], hi); mine += sh.s[k]; }
-    int incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    sh.start = incl - mine;
-    return sh;
+    return last - static_cast<int>(found & static_cast<uint32_t>(last));
 }
 
 // ---- warp-level tensor-core MMAs (m16n8k32 INT8 / m16n8k16 FP16, FP32 or INT32 accumulators) ----------
@@ -141,29 +128,14 @@ decode_kernel(const DecodeParams prm) {
     const int hk = blockIdx.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t = lane & 3;
-    int split = blockIdx.x, b = blockIdx.z, row_splits = prm.n_splits;
-    if (prm.balanced) {      // gridDim.x CTAs per KV head, shared out over the sequences
-        const Shares sh = share_out<T>(prm.cache_len_raw, prm.B, prm.max_len, prm.n_ctas);
-        int found = -1, part = 0, n = 0, start = sh.start;
-#pragma unroll
-        for (int k = 0; k < kShareRows; ++k) {
-            const int at = static_cast<int>(blockIdx.x) - start;
-            if (at >= 0 && at < sh.s[k]) { found = lane * sh.K + k; part = at; n = sh.s[k]; }
-            start += sh.s[k];
-        }
-        const unsigned who = __ballot_sync(0xffffffffu, found >= 0);
-        if (who == 0u) return;                                    // a CTA left over
-        const int src = __ffs(who) - 1;
-        b = __shfl_sync(0xffffffffu, found, src);
-        split = __shfl_sync(0xffffffffu, part, src);
-        row_splits = __shfl_sync(0xffffffffu, n, src);
-    }
+    const int split = blockIdx.x;
     // (lengths live on the device and cannot be checked by the host: out-of-range values are clamped.  This grid may run
     // beside the prepare kernel, so it clamps the caller's array itself, and waits for that kernel only where it writes
     // the status record.)
+    const int b = prm.by_length ? nth_longest<T>(prm.cache_len_raw, prm.B, prm.max_len, blockIdx.z) : blockIdx.z;
     const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
-    const int per_split = (n_tiles + row_splits - 1) / row_splits;
+    const int per_split = (n_tiles + prm.n_splits - 1) / prm.n_splits;
     const int t0 = split * per_split, t1 = min(n_tiles, t0 + per_split);
 
     extern __shared__ __align__(128) uint8_t ring[];   // n_stages x (K tile | V tile)
@@ -520,9 +492,7 @@ decode_kernel(const DecodeParams prm) {
                 z += red[w][r][D + 1] * wgt;
             }
         }
-        // partial result of this CTA: balanced, number blockIdx.x of its query head's pool; else [sequence, head, split]
-        const int64_t row = prm.balanced ? static_cast<int64_t>(hk * R + r) * prm.n_ctas + blockIdx.x
-                                         : (static_cast<int64_t>(b) * prm.Hq + hk * R + r) * prm.n_splits + split;
+        const int64_t row = (static_cast<int64_t>(b) * prm.Hq + hk * R + r) * prm.n_splits + split;
         prm.o_part[row * D + e] = o;
         if (e == 0) { prm.m_part[row] = m; prm.z_part[row] = z; }
     }
@@ -536,28 +506,15 @@ template <int D>
 __global__ void __launch_bounds__(D)
 decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ m_part,
                     const float* __restrict__ z_part, int n_splits, __half* __restrict__ out,
-                    float* __restrict__ lse, const int32_t* __restrict__ cache_len, int B, int max_len, int Hq) {
-    const int64_t row = blockIdx.x;
-    int64_t first = row * n_splits;      // of the row's partial results
-    if (cache_len != nullptr) {          // balanced warp-level form: n_splits is the size of a query head's pool
-        const Shares sh = share_out<kChunk<D>>(cache_len, B, max_len, n_splits);
-        const int b = static_cast<int>(row) / Hq, hq = static_cast<int>(row) - b * Hq;
-        int n = 0, start = sh.start;
-#pragma unroll
-        for (int k = 0; k < kShareRows; ++k) {
-            if (k < b % sh.K) start += sh.s[k];
-            if (k == b % sh.K) n = sh.s[k];
-        }
-        first = static_cast<int64_t>(hq) * n_splits + __shfl_sync(0xffffffffu, start, b / sh.K);
-        n_splits = __shfl_sync(0xffffffffu, n, b / sh.K);
-    }
+                    float* __restrict__ lse) {
     ptx::griddep_wait();   // (when launched as a programmatic dependent of the step kernel)
+    const int64_t row = blockIdx.x;
     const int e = threadIdx.x, lane = e & 31;
     float m = -INFINITY, z = 0.f, o = 0.f;
     for (int s0 = 0; s0 < n_splits; s0 += 32) {
         const int s = s0 + lane;
-        const float ms = s < n_splits ? m_part[first + s] : -INFINITY;
-        const float zs = s < n_splits ? z_part[first + s] : 0.f;
+        const float ms = s < n_splits ? m_part[row * n_splits + s] : -INFINITY;
+        const float zs = s < n_splits ? z_part[row * n_splits + s] : 0.f;
         float mc = ms;
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, d));
@@ -568,7 +525,7 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
         const float zw = ms == -INFINITY ? 0.f : zs * w;
         z *= back; o *= back; m = m_new;
         const int cnt = min(32, n_splits - s0);
-        const float* src = o_part + (first + s0) * D + e;
+        const float* src = o_part + (row * n_splits + s0) * D + e;
 #pragma unroll 8
         for (int i = 0; i < cnt; ++i) {
             const float wi = __shfl_sync(0xffffffffu, w, i);
@@ -582,7 +539,7 @@ decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ 
 
 // Step and merge overlap the tail of the kernel before them (programmatic dependent launch).
 template <int D>
-int launch_merge(const DecodeParams& prm, int n_splits, bool shared, __half* out, float* lse, cudaStream_t stream) {
+int launch_merge(const DecodeParams& prm, int n_splits, __half* out, float* lse, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(prm.B * prm.Hq); cfg.blockDim = dim3(D); cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -591,8 +548,7 @@ int launch_merge(const DecodeParams& prm, int n_splits, bool shared, __half* out
     cfg.attrs = attr; cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_merge_kernel<D>, static_cast<const float*>(prm.o_part),
                                              static_cast<const float*>(prm.m_part), static_cast<const float*>(prm.z_part),
-                                             n_splits, out, lse, shared ? prm.cache_len_raw : static_cast<const int32_t*>(nullptr),
-                                             prm.B, prm.max_len, prm.Hq);
+                                             n_splits, out, lse);
     g_launch_count.fetch_add(1);
     return static_cast<int>(e);
 }
@@ -604,7 +560,7 @@ int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t st
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
     if (e != cudaSuccess) return static_cast<int>(e);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = prm.balanced ? dim3(prm.n_ctas, prm.Hk) : dim3(prm.n_splits, prm.Hk, prm.B);
+    cfg.gridDim = dim3(prm.n_splits, prm.Hk, prm.B);
     cfg.blockDim = dim3(kDecodeThreads); cfg.dynamicSmemBytes = kRingBytes; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -613,7 +569,7 @@ int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t st
     e = cudaLaunchKernelEx(&cfg, kernel, prm);
     g_launch_count.fetch_add(1);
     if (e != cudaSuccess) return static_cast<int>(e);
-    return launch_merge<D>(prm, prm.balanced ? prm.n_ctas : prm.n_splits, prm.balanced != 0, out, lse, stream);
+    return launch_merge<D>(prm, prm.n_splits, out, lse, stream);
 }
 
 template <int D, int RT>
@@ -694,23 +650,21 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
                 g->balanced = 1; g->n_ctas = static_cast<int>(ctas); g->split_cap = row_cap;
             }
         } else {
-            // at most two full waves of two CTAs per SM over the whole batch (measured: more splits cost
-            // more in per-CTA set-up and merge than they gain, and a third, partial wave idles a quarter
-            // of the GPU), at least two key tiles per split
-            const int64_t want = (148 * 2 * 2) / (static_cast<int64_t>(p->batch) * p->heads_kv);
+            // Two CTAs per SM, in one wave or -- batches of long sequences -- two (a third, partial one idles a quarter of the
+            // GPU), with at least two kernel tiles per split.  A CTA costs its set-up, drain and partial result, which one
+            // wave pays once; two waves of shorter CTAs even out unequal lengths.  The line is where a CTA of the second
+            // form has twelve kernel tiles.  us in one wave and in two, lengths equal / uniform in [0, max]: d = 64,
+            // 50 rows x 5000 keys (3.6 tiles) 28 / 26 and 32 / 30; 72 x 8000 (7.9) 36 / 32 and 42 / 32; 200 x 3000 (12)
+            // 46 / 42 and 50 / 30; 64 x 16384 (14) 60 / 48 and 64 / 40; 128 x 8192 (16) 58 / 52 and 64 / 42; d = 128:
+            // 48 x 4000 (5.2) 32 / 26 and 38 / 30; 32 x 12000 (10) 46 / 36 and 56 / 38; 64 x 16384 (28) 101 / 75 and
+            // 101 / 60.  One sequence has nothing to even out: 8 rows x 65536 keys 44 and 56.
+            const int64_t rows = static_cast<int64_t>(p->batch) * p->heads_kv, wave = 2 * kDecodeWave;
+            const int k_tiles = static_cast<int>(ceil_div(p->max_len, p->head_dim == 64 ? kChunk<64> : kChunk<128>));
+            int64_t want = 2 * wave / rows;
+            if (p->batch == 1 || k_tiles < 12 * (want < 1 ? 1 : want)) want = wave / rows;
+            const int cap = k_tiles / 2 > 0 ? k_tiles / 2 : 1;
+            if (want > cap) want = cap;
             splits = static_cast<int>(want < 1 ? 1 : want);
-            const int cap = g->n_blk / 2 > 0 ? g->n_blk / 2 : 1;
-            if (splits > cap) splits = cap;
-            // No more partial results than that, but shared out over the sequences by their cache lengths: one wave of
-            // two CTAs per SM where that is at least two per sequence, else two.  (16 x 8 rows of up to 8K keys, d = 64:
-            // 42 us; with two waves, whose CTAs are shorter and start one behind the other, 48.)
-            if (p->batch <= kMaxShared) {
-                const int64_t wave = 2 * kDecodeWave / p->heads_kv;
-                int64_t pool = p->batch * 2 <= wave ? wave : 2 * wave;
-                if (pool > static_cast<int64_t>(p->batch) * splits) pool = static_cast<int64_t>(p->batch) * splits;
-                if (pool < p->batch) pool = p->batch;
-                g->balanced = 1; g->n_ctas = static_cast<int>(pool);
-            }
         }
     }
     if (splits > g->n_blk) splits = g->n_blk;
@@ -756,6 +710,7 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     prm.tile_n = p->tile_n;
     prm.n_parts = g.n_parts; prm.balanced = g.balanced; prm.n_rows = p->batch * p->heads_kv;
     prm.n_ctas = g.n_ctas; prm.split_cap = g.split_cap;
+    prm.by_length = p->batch > 1 && p->batch <= kMaxSorted ? 1 : 0;
     const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf(static_cast<float>(p->head_dim));
     prm.scale_log2 = scale * kLog2e;
     prm.q = static_cast<const __half*>(q_f16);
@@ -787,7 +742,7 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
         // the tcgen05 form of the step (decode_umma.cu), then the same merge
         rc = launch_decode_umma(R, prm, s);
         if (rc) return rc;
-        return launch_merge<128>(prm, g.n_parts, false, out, lse, s);
+        return launch_merge<128>(prm, g.n_parts, out, lse, s);
     }
     if (p->head_dim == 128 && p->tile_n == 64) return launch_r<128, 64>(R, prm, out, lse, s);
     if (p->head_dim == 64 && p->tile_n == 128) return launch_r<64, 128>(R, prm, out, lse, s);

@@ -12,10 +12,10 @@ struct DecodeParams {
     int B, Hq, Hk, max_len, G, nb, W, n_splits, n_blk;
     int tile_n;      // tokens per scale block and per routing key tile (a multiple of the kernel's chunk)
     int n_parts;     // partial results per query head in the workspace
-    // Automatic split count; n_splits is then not used.  tcgen05 form: n_ctas CTAs (one wave or two) are shared out over
-    // the n_rows = B * Hk rows by their cost, at most split_cap to a row (n_parts = 2 * split_cap).  Warp-level form:
-    // n_ctas CTAs and partial results per KV / query head are shared out over the sequences by their cache lengths.
+    // tcgen05 form, automatic split count: n_ctas CTAs (one wave or two) are shared out over the n_rows = B * Hk rows by
+    // their cost, at most split_cap to a row (n_parts = 2 * split_cap); n_splits is then not used
     int balanced, n_rows, n_ctas, split_cap;
+    int by_length;   // warp-level form: the grid takes the sequences longest first
     float scale_log2;
     const __half* q;
     const __half* k16;

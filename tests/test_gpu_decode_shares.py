@@ -1,10 +1,12 @@
-"""Warp-level decode form: two 64-key routing tiles per kernel tile, and partial results shared out over sequences of
-unequal length (library-chosen splits) -- one to eight sequences per lane of the warp that shares them out, lengths at
-the edges of kernel and routing tiles, more sequences than CTAs of a wave."""
+"""Warp-level decode form: two 64-key routing tiles per kernel tile, and a grid that takes sequences of unequal length
+longest first -- one to eight sequences per lane of the warp that orders them, lengths at the edges of kernel and routing
+tiles, more sequences than are ordered; a sequence's result does not depend on the sequences beside it.  The tcgen05
+form with CTAs shared out over the rows, two waves of them."""
 import numpy as np
 import pytest
+import torch
 
-from tests.test_gpu_decode import _case, _check
+from tests.test_gpu_decode import _case, _check, _gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -21,9 +23,34 @@ def test_unequal_lengths(B, Hq, Hk, L, G, splits, d, tile):
     _check(q, k, v, route, lens, tile, G, n_splits=splits)
 
 
-def test_more_sequences_than_are_shared_out():
+def test_more_sequences_than_are_ordered():
     q, k, v, route, lens = _case(300, 1, 1, 200, 64, 64, 1, seed=3, lens=np.arange(300) % 201)
     _check(q, k, v, route, lens, 64, 1)
+
+
+@pytest.mark.parametrize("splits", [0, -1, 5])
+@pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (128, 64), (128, 128)])
+@pytest.mark.parametrize("B", [6, 40])
+def test_a_sequence_does_not_depend_on_the_lengths_beside_it(B, d, tile, splits):
+    """Same bits whatever the other sequences' lengths are, and in a repeated call; every length 0 included.  (In the
+    tcgen05 form -1 shares CTAs out by the lengths.)"""
+    if (d, tile, splits) == (128, 128, -1):
+        splits = 1
+    L = 1500
+    first = np.random.default_rng(B).integers(1, L + 1, B)
+    keep = np.arange(B) % 3 == 0
+    runs = []
+    for others in (first, first, np.full(B, L), np.zeros(B, np.int64), first[::-1]):
+        lens = np.where(keep, first, others)
+        q, k, v, route, lens = _case(B, 4, 2, L, d, tile, 2, seed=5, lens=lens)
+        res, _ = _gpu(q, k, v, route, lens, tile, 2, n_splits=splits)
+        runs.append((res["out"][keep].cpu(), res["lse"][keep].cpu()))
+    for out, lse in runs[1:]:
+        assert torch.equal(out, runs[0][0]) and torch.equal(lse, runs[0][1])
+    q, k, v, route, lens = _case(B, 4, 2, L, d, tile, 2, seed=5, lens=np.zeros(B))
+    _check(q, k, v, route, np.append(lens[:-1], 1).astype(np.int32), tile, 2, n_splits=splits)
+    res, _ = _gpu(q, k, v, route, lens, tile, 2, n_splits=splits)
+    assert not res["out"].any() and torch.isneginf(res["lse"]).all()
 
 
 @pytest.mark.parametrize("B,Hq,Hk,L,G", [(10, 16, 8, 1000, 1), (40, 8, 4, 400, 2), (80, 2, 2, 300, 1)])
