@@ -653,10 +653,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             if (!ok) break;
             if (n < nkv) {
                 const uint32_t e = sched(n);
-                uint32_t r = SUB ? (e >> (4 * h + 2 * t + rh)) & 1u : (e >> t) & 1u;
-                // keys above the diagonal of these rows: all masked, so the factor is one that is finite (delta_K is
-                // not where a key of the block is not)
-                if (SUB && 2 * n + h > (t ? dB : dA) + rh) r = 0u;
+                const uint32_t r = SUB ? (e >> (4 * h + 2 * t + rh)) & 1u : (e >> t) & 1u;
                 if (lane < kNumSc + (VS ? 2 : 0))
                     sc_s[(n % C::kScSlots) * C::kScStride + lane] = lane < kNumSc ? factor(r, dq, cur) : cur;
             }
@@ -870,19 +867,11 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 }
             };
             // O_t (+)= P_t V_j over the keys of half h, with P in tensor memory (two FP16 per 32-bit
-            // column, at the start of its own half of S_t).  `above` (D = 64, never the first step): the keys lie above
-            // the diagonal of the first row half.  Its P is 0 there, but 0 times a value that is not finite is not, so
-            // its lanes are switched off: a row sees V of no key beyond its own 64-key tile.
-            auto issue_pv = [&](int t, int h, uint32_t sv, uint32_t accumulate, bool above) {
+            // column, at the start of its own half of S_t)
+            auto issue_pv = [&](int t, int h, uint32_t sv, uint32_t accumulate) {
                 const uint32_t d_tmem = tmem_base + 2 * C::kSCols + t * C::kOCols;
                 const uint32_t a_tmem = tmem_base + t * C::kSCols + h * TH;
                 const uint32_t b_lo = ring_lo_v + sv * kChunkLo + h * (TH / 16) * 128;
-                if (SUB && above) {
-#pragma unroll
-                    for (int k = 0; k < TH / 16; ++k)
-                        ptx::mma_f16_ts_lanes<true>(d_tmem, a_tmem + k * 8, b_lo + k * 128, kHi16, kIdescPV, 0xffffffffu, 0u);
-                    return;
-                }
                 ptx::mma_f16_ts(d_tmem, a_tmem, b_lo, kHi16, kIdescPV, accumulate);
 #pragma unroll
                 for (int k = 1; k < TH / 16; ++k)
@@ -925,7 +914,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                         if (SUB && 2 * j + h >= u_t) break;
                         if (!wait_bar(cx, bar_p(t, h), j & 1, kRoleMma, j, kBarP)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
-                        issue_pv(t, h, sv, (j > 0 || h > 0) ? 1u : 0u, SUB && 2 * j + h > (t ? dB : dA));
+                        issue_pv(t, h, sv, (j > 0 || h > 0) ? 1u : 0u);
                         if (2 * j + h == u_t - 2) ptx::mma_commit(bar_pv(t));   // the last-but-one PV (a rescale in the last step waits for it)
                         if (2 * j + h == u_t - 1) ptx::mma_commit(bar_o(t));
                         if (2 * (j + 1) + h < u_t) {
@@ -967,7 +956,12 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             const int role = t ? kRoleSoftmaxB : kRoleSoftmaxA;
             // this warp's scaling factors in the ring (see there)
             const uint32_t sc0 = SUB ? (2 * t + rh) * (KH ? 2 : 1) : t;
-            const int n_steps = t ? uB : uA;
+            const int n_all = t ? uB : uA;         // steps of the tile
+            // D = 64: the keys of the tile's last step lie above the diagonal of its first row half.  Those rows are done
+            // a step earlier and take their O before that step's PV: a probability of 0 there would still meet V, and 0
+            // times a value that is not finite is not 0 (nor is a masked score times such a block's scale).
+            const bool early = SUB && rh == 0 && n_all > d_t + 1;
+            const int n_steps = early ? d_t + 1 : n_all;
             // One step = one half (TH key columns) of a score tile: while the warps of this tile work on one half of
             // S_t, the tensor pipe runs the PV of the previous half and the QK^T of the next one into the other
             // half.  u = 2*j + h.
@@ -1110,7 +1104,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     // The issuer puts the QK^T of step u+1 behind PV(u-1) and commits both to "S(u+1) ready",
                     // so that barrier -- the one the next step waits on anyway -- says PV(u-1) has retired; the
                     // last step has no successor and waits on the commit behind the last-but-one PV instead.
-                    if (u + 1 < n_steps) ok = wait_bar(cx, bar_s(t, h ^ 1), ((u + 1) >> 1) & 1, role, j, kBarS);
+                    if (u + 1 < n_all) ok = wait_bar(cx, bar_s(t, h ^ 1), ((u + 1) >> 1) & 1, role, j, kBarS);
                     else ok = wait_bar(cx, bar_pv(t), 0, role, j, kBarPV);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
@@ -1135,12 +1129,25 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             }
 
             if (ok) {
-                ok = wait_bar(cx, bar_o(t), 0, role, (n_steps + 1) >> 1, kBarO);
+                // (early: the last-but-one PV is this row half's last)
+                ok = early ? wait_bar(cx, bar_pv(t), 0, role, (n_steps + 1) >> 1, kBarPV)
+                           : wait_bar(cx, bar_o(t), 0, role, (n_steps + 1) >> 1, kBarO);
                 ok = __all_sync(0xffffffffu, ok);
             }
             if (ok) {
                 // Finalise (Sec. 3.1): O = O~ / z in FP16; LSE = m + ln z.
                 ptx::tc_fence_after_sync();
+                uint32_t o[SUB ? D / 32 : 1][16];
+                if constexpr (SUB) {
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c) ptx::tmem_ld16x256_x4(t_o + c * 32, o[c]);
+#pragma unroll
+                    for (int c = 0; c < D / 32; ++c) ptx::tmem_wait_ld_dep(o[c]);
+                    if (early) {       // the step above the diagonal may have its PV (P of these rows: whatever is there)
+                        ptx::tc_fence_before_sync();
+                        ptx::mbar_arrive(bar_p(t, (d_t + 1) & 1));
+                    }
+                }
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const float z_row = quad_sum(z[k]);
@@ -1158,15 +1165,17 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 const bool odd = lane & 1, upper = lane & 2;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {
-                    uint32_t o[16];
-                    ptx::tmem_ld16x256_x4(t_o + c * 32, o);
-                    ptx::tmem_wait_ld_dep(o);
+                    uint32_t (&oc)[16] = o[SUB ? c : 0];
+                    if constexpr (!SUB) {
+                        ptx::tmem_ld16x256_x4(t_o + c * 32, oc);
+                        ptx::tmem_wait_ld_dep(oc);
+                    }
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         uint32_t w[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
-                            w[i] = pack_half2(__uint_as_float(o[4 * i + 2 * k]) * z[k], __uint_as_float(o[4 * i + 2 * k + 1]) * z[k]);
+                            w[i] = pack_half2(__uint_as_float(oc[4 * i + 2 * k]) * z[k], __uint_as_float(oc[4 * i + 2 * k + 1]) * z[k]);
 #pragma unroll
                         for (int i = 0; i < 4; i += 2) {      // columns <-> lanes 0, 1 of every pair
                             const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? w[i] : w[i + 1], 1);
