@@ -307,7 +307,9 @@ typedef struct tilemix_decode {
                             * the tcgen05 form with batch * heads_kv <= 148 the CTAs of one wave (two, with more than
                             * 74 rows) are shared out so that the largest number of cache bytes a CTA reads is as
                             * small as it can be (a row gets clamp(ceil(bytes / tau), 1, cap) CTAs for the smallest
-                            * tau that fits); elsewhere -1 means 0.  Except in that shared-out form, what a sequence's
+                            * tau that fits); elsewhere -1 means 0.  A split is a whole number of 128-key pieces of
+                            * the cache (64-key ones at head_dim 128 with 64-key tiles), and a count above their
+                            * number means that number.  Except in that shared-out form, what a sequence's
                             * result is does not depend on the lengths beside it. */
     float softmax_scale;   /* <= 0 means 1/sqrt(head_dim)                                   */
 } tilemix_decode_t;

@@ -625,6 +625,7 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
     const bool balance = p->n_splits == -1;
     int splits = balance ? 0 : p->n_splits;
     const bool umma = p->head_dim == 128 && p->tile_n == 128;   // the tcgen05 form of the step (decode_umma.cu)
+    const int k_tiles = umma ? g->n_blk : static_cast<int>(ceil_div(p->max_len, p->head_dim == 64 ? kChunk<64> : kChunk<128>));
     g->balanced = 0; g->n_ctas = 0; g->split_cap = 0;
     if (splits == 0) {
         if (umma) {
@@ -659,7 +660,6 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
             // 48 x 4000 (5.2) 32 / 26 and 38 / 30; 32 x 12000 (10) 46 / 36 and 56 / 38; 64 x 16384 (28) 101 / 75 and
             // 101 / 60.  One sequence has nothing to even out: 8 rows x 65536 keys 44 and 56.
             const int64_t rows = static_cast<int64_t>(p->batch) * p->heads_kv, wave = 2 * kDecodeWave;
-            const int k_tiles = static_cast<int>(ceil_div(p->max_len, p->head_dim == 64 ? kChunk<64> : kChunk<128>));
             int64_t want = 2 * wave / rows;
             if (p->batch == 1 || k_tiles < 12 * (want < 1 ? 1 : want)) want = wave / rows;
             const int cap = k_tiles / 2 > 0 ? k_tiles / 2 : 1;
@@ -669,6 +669,7 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
     }
     if (splits > g->n_blk) splits = g->n_blk;
     if (splits > 65535) return TILEMIX_ERR_UNSUPPORTED;
+    if (splits > k_tiles) splits = k_tiles;      // a split is whole kernel tiles: more of them would only be empty CTAs
     g->n_splits = splits;
     g->n_parts = umma ? 2 * (g->balanced ? g->split_cap : splits) : splits;
     const size_t rows = static_cast<size_t>(p->batch) * p->heads_q * g->n_parts;

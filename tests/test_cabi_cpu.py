@@ -259,3 +259,13 @@ def test_chunk_v8_host_side_validation(lib):
     otf = b.problem(1, 4, 2, 256, 128, 128, 128, flags=b.QUANT_ON_THE_FLY)
     assert call(otf, 1024, args) == b.ERR_UNSUPPORTED
     assert lib.tilemix_attention_fwd_chunk_v8(None, 1024, *args, one, need, None) == b.ERR_NULL
+
+
+def test_a_decode_split_is_whole_kernel_tiles(lib):
+    """head_dim 64: kernel tiles of 128 keys, also with 64-key routing tiles; a larger count than there are means theirs."""
+    size = lambda n, d=64, tile=64, L=4096: b.tilemix_decode_workspace_size(b.decode_problem(2, 4, 2, d, L, tile, n_splits=n))  # noqa: E731
+    assert size(31) < size(32) == size(33) == size(64) == size(1000)
+    assert size(1000, L=4097) == size(33, L=4097) > size(1000)
+    assert size(63, d=128) < size(64, d=128) == size(1000, d=128)
+    # a count that the grid cannot hold stays refused, whatever its splits would have been
+    assert size(70000, L=1 << 23) == 0 and size(40000, L=1 << 23) > 0

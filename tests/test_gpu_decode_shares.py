@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("d,tile", [(64, 64), (64, 128), (128, 64)])
 @pytest.mark.parametrize("B,Hq,Hk,L,G,splits", [(1, 2, 1, 700, 1, 0), (5, 4, 2, 1500, 3, 0), (33, 4, 4, 400, 1, -1), (100, 8, 1, 300, 2, 0),
-                                                (200, 2, 2, 260, 1, 0), (4, 2, 1, 900, 1, 3)])
+                                                (200, 2, 2, 260, 1, 0), (4, 2, 1, 900, 1, 3), (4, 2, 1, 900, 1, 1000)])
 def test_unequal_lengths(B, Hq, Hk, L, G, splits, d, tile):
     rng = np.random.default_rng(B + L)
     lens = rng.integers(0, L + 1, B)
