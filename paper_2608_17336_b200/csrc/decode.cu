@@ -130,8 +130,8 @@ decode_kernel(const DecodeParams prm) {
     const int g = lane >> 2, t = lane & 3;
     const int split = blockIdx.x;
     // (lengths live on the device and cannot be checked by the host: out-of-range values are clamped.  This grid may run
-    // beside the prepare kernel, so it clamps the caller's array itself, and waits for that kernel only where it writes
-    // the status record.)
+    // beside the prepare kernel, so it clamps the caller's array itself, and waits for that kernel before it writes the
+    // status record or ends.)
     const int b = prm.by_length ? nth_longest<T>(prm.cache_len_raw, prm.B, prm.max_len, blockIdx.z) : blockIdx.z;
     const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
@@ -438,8 +438,10 @@ decode_kernel(const DecodeParams prm) {
 
     // ---- merge of the eight warps, then (m, z, O~) of this split to the workspace --------------------
     __syncthreads();   // every warp is out of the ring (all copies it waited for have landed)
+    // The prepare kernel has completed before this grid does: the merge kernel waits for this grid only, and what the
+    // stream runs behind it may read the status record or use the workspace again.
+    ptx::griddep_wait();
     if (*reinterpret_cast<volatile int*>(&abort_flag)) {
-        ptx::griddep_wait();
         if (tid == 0 && atomicCAS(&prm.status[0], 0, TILEMIX_ERR_DEVICE_TIMEOUT) == 0) {
             prm.status[1] = 16; prm.status[2] = t0; prm.status[3] = 0;
         }

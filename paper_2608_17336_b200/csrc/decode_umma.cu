@@ -153,6 +153,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&sh.tmem_base);
     auto leave = [&]() {                  // early exits: tensor memory goes back first
+        ptx::griddep_wait();              // (see the end of the kernel)
         __syncthreads();
         if (warp == kProducerWarp) ptx::tmem_dealloc(tmem_base, kTmemCols);
     };
@@ -221,7 +222,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     }
     // This grid may run beside the prepare kernel (programmatic dependent launch): it takes the length from the
     // caller's array with the same clamp, and waits for the prepare kernel (which clears the status record) only
-    // where it is about to write that record.
+    // where it is about to write that record, and at its end.
     const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
     const uint32_t* wrow = row_words(b, hk);
@@ -722,6 +723,9 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     }
 
     // ---- every role is out of its loop ---------------------------------------------------------------------
+    // The prepare kernel has completed before this grid does: the merge kernel waits for this grid only, and what the
+    // stream runs behind it may read the status record or use the workspace again.
+    ptx::griddep_wait();
     __syncthreads();
     if (*abort_flag && warp == kProducerWarp && lane == 0) {
         // the copies still in flight land before this CTA's shared memory is given back
