@@ -314,7 +314,7 @@ typedef struct tilemix_decode {
     float softmax_scale;   /* <= 0 means 1/sqrt(head_dim)                                   */
 } tilemix_decode_t;
 
-/* Bytes of `workspace` for tilemix_decode_int8kv: the status record, the clamped copy of the cache lengths
+/* Bytes of `workspace` for tilemix_decode_int8kv: the status record, a reserved area of four bytes per sequence
  * and the partial results of the splits (0 on an invalid problem). */
 size_t tilemix_decode_workspace_size(const tilemix_decode_t* p);
 /*   q_f16      FP16 [B, Hq, d]
@@ -330,9 +330,8 @@ size_t tilemix_decode_workspace_size(const tilemix_decode_t* p);
  *   out_f16    FP16 [B, Hq, d];  lse nullable FP32 [B, Hq]
  *   q_i8_out / q_scale_out  nullable INT8 [B, Hq, d] / FP32 [B, Hq]: the quantised query the
  *              kernel used (for checking)
- * Three kernels are enqueued on `stream` (preparation of the lengths and the status record, the step over the
- * splits, the merge; in the tcgen05 form the last two are programmatic dependent launches, so that their set-up
- * overlaps the kernel before them).  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
+ * Three kernels are enqueued on `stream` (one that clears the status record, the step over the splits, the merge;
+ * the last two are programmatic dependent launches, so that their set-up overlaps the kernel before them).  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
  * kernel itself found (a bounded wait that ran out, or the missing FP16 cache above). */
 int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const void* k_f16,
                           const int8_t* k_i8, const float* k_scale, const int8_t* v_i8,

@@ -132,8 +132,8 @@ decode_kernel(const DecodeParams prm) {
     // (lengths live on the device and cannot be checked by the host: out-of-range values are clamped.  This grid may run
     // beside the prepare kernel, so it clamps the caller's array itself, and waits for that kernel before it writes the
     // status record or ends.)
-    const int b = prm.by_length ? nth_longest<T>(prm.cache_len_raw, prm.B, prm.max_len, blockIdx.z) : blockIdx.z;
-    const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
+    const int b = prm.by_length ? nth_longest<T>(prm.cache_len, prm.B, prm.max_len, blockIdx.z) : blockIdx.z;
+    const int len = min(max(prm.cache_len[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
     const int per_split = (n_tiles + prm.n_splits - 1) / prm.n_splits;
     const int t0 = split * per_split, t1 = min(n_tiles, t0 + per_split);
@@ -589,16 +589,14 @@ constexpr size_t kDecodeStatusBytes = 256;   // status record of the bounded wai
 constexpr int kDecodeWave = 148;             // CTAs of one wave of the tcgen05 form (one per SM)
 constexpr int kDecodeBalanceRows = 160;      // rows of a batch whose splits that kernel can balance
 
-// Before the step: clears the status record and copies the cache lengths, clamped to [0, max_len], into the
-// workspace (they live on the device, so the host cannot check them; the step itself reads the copy).
-__global__ void decode_prepare_kernel(const int32_t* __restrict__ cache_len, int B, int max_len, int* status,
-                                      int32_t* __restrict__ len_out) {
-    ptx::griddep_launch_dependents();   // the step kernel may set itself up meanwhile; it waits before it reads these
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 4) status[i] = 0;
-    if (i < B) len_out[i] = min(max(cache_len[i], 0), max_len);
+// Before the step: clears the status record.  (The cache lengths live on the device, so the host cannot check them: the
+// step clamps each to [0, max_len] as it reads it.)
+__global__ void decode_prepare_kernel(int* status) {
+    ptx::griddep_launch_dependents();   // the step kernel may start meanwhile; it waits before it writes the record or ends
+    if (threadIdx.x < 4) status[threadIdx.x] = 0;
 }
 
+// Reserved behind the status record (it held a copy of the lengths): the size of a workspace stays what it was.
 size_t decode_len_bytes(int B) { return (static_cast<size_t>(B) * sizeof(int32_t) + 255) / 256 * 256; }
 
 struct DecodeGeometry {
@@ -710,7 +708,6 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     DecodeParams prm{};
     prm.B = p->batch; prm.Hq = p->heads_q; prm.Hk = p->heads_kv; prm.max_len = p->max_len; prm.G = p->group;
     prm.nb = p->mask_batch; prm.W = g.W; prm.n_splits = g.n_splits; prm.n_blk = g.n_blk;
-    prm.tile_n = p->tile_n;
     prm.n_parts = g.n_parts; prm.balanced = g.balanced; prm.n_rows = p->batch * p->heads_kv;
     prm.n_ctas = g.n_ctas; prm.split_cap = g.split_cap;
     prm.by_length = p->batch > 1 && p->batch <= kMaxSorted ? 1 : 0;
@@ -723,9 +720,7 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     prm.status = static_cast<int*>(workspace);
     prm.wait_limit_ns = g_wait_limit_ns.load();
     prm.test_drop_tile = g_test_drop.load() == 2 ? 1 : -1;
-    int32_t* len_ws = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + kDecodeStatusBytes);
-    prm.cache_len = len_ws;
-    prm.cache_len_raw = cache_len;
+    prm.cache_len = cache_len;
     uint8_t* ws = static_cast<uint8_t*>(workspace) + kDecodeStatusBytes + decode_len_bytes(p->batch);
     prm.o_part = reinterpret_cast<float*>(ws);
     prm.m_part = reinterpret_cast<float*>(ws + g.o_bytes);
@@ -734,13 +729,10 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int R = p->heads_q / p->heads_kv;
     __half* out = static_cast<__half*>(out_f16);
-    const int prep_threads = p->batch > 4 ? p->batch : 4;
-    decode_prepare_kernel<<<(prep_threads + 255) / 256, 256, 0, s>>>(cache_len, p->batch, p->max_len, prm.status, len_ws);
+    decode_prepare_kernel<<<1, 32, 0, s>>>(prm.status);
     g_launch_count.fetch_add(1);
     cudaError_t pe = cudaGetLastError();
     if (pe != cudaSuccess) return static_cast<int>(pe);
-    // keys are streamed and processed one routing tile at a time (64-key chunks with a deeper ring
-    // were slower: the per-chunk barriers cost more than the extra bytes in flight gain)
     if (p->head_dim == 128 && p->tile_n == 128) {
         // the tcgen05 form of the step (decode_umma.cu), then the same merge
         rc = launch_decode_umma(R, prm, s);

@@ -10,7 +10,6 @@ namespace tilemix {
 
 struct DecodeParams {
     int B, Hq, Hk, max_len, G, nb, W, n_splits, n_blk;
-    int tile_n;      // tokens per scale block and per routing key tile (a multiple of the kernel's chunk)
     int n_parts;     // partial results per query head in the workspace
     // tcgen05 form, automatic split count: n_ctas CTAs (one wave or two) are shared out over the n_rows = B * Hk rows by
     // their cost, at most split_cap to a row (n_parts = 2 * split_cap); n_splits is then not used
@@ -24,8 +23,7 @@ struct DecodeParams {
     const int8_t* v8;
     const float* v_scale;
     const uint32_t* words;
-    const int32_t* cache_len;       // clamped copy in the workspace (written by the prepare kernel)
-    const int32_t* cache_len_raw;   // the caller's array
+    const int32_t* cache_len;       // the caller's array (device memory; read with a clamp to [0, max_len])
     float* o_part;   // [B, Hq, n_parts, D]
     float* m_part;   // [B, Hq, n_parts]
     float* z_part;

@@ -107,14 +107,14 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         return prm.words != nullptr ? prm.words + (static_cast<int64_t>(prm.nb == 1 ? 0 : bb) * prm.Hk + hh) * prm.W : nullptr;
     };
     auto row_groups = [&](int bb) -> int {
-        const int l = min(max(prm.cache_len_raw[bb], 0), prm.max_len);
+        const int l = min(max(prm.cache_len[bb], 0), prm.max_len);
         return ((l + T - 1) / T + prm.G - 1) / prm.G;
     };
     auto word_cost = [&](const uint32_t* wr, int w, int nb) -> int {
         const uint32_t bits = wr != nullptr ? wr[w] & (nb >= 32 ? 0xffffffffu : ((1u << nb) - 1u)) : 0u;
         return 3 * nb - __popc(bits);
     };
-    // Balanced splits (one wave of CTAs over a batch of at most kMaxRows rows): thread i adds up the cost of row i.
+    // Balanced splits (one wave of CTAs, or two, over a batch of at most kMaxRows rows): thread i adds up the cost of row i.
     if (prm.balanced && tid < prm.n_rows) {
         const int bb = tid / prm.Hk;
         const uint32_t* wr = row_words(bb, tid - bb * prm.Hk);
@@ -158,8 +158,8 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         if (warp == kProducerWarp) ptx::tmem_dealloc(tmem_base, kTmemCols);
     };
     // ---- which part of which row -------------------------------------------------------------------------------
-    // Uniform form: the grid is (splits, KV heads, sequences).  Balanced form: gridDim.x CTAs, one per SM, are
-    // shared out over the rows so that the largest cost of a CTA is as small as it can be -- with one wave the
+    // Uniform form: the grid is (splits, KV heads, sequences).  Balanced form: gridDim.x CTAs, one or two per SM one
+    // after the other, are shared out over the rows so that the largest cost of a CTA is as small as it can be -- the
     // CTA with the most bytes ends last, and rows differ (cache lengths, FP16-routed groups).  Row i gets
     // s_i = clamp(ceil(c_i / tau), 1, cap) CTAs for the smallest tau whose total fits the grid; CTAs left over
     // leave.  Every CTA finds the same tau (one warp, a binary search over at most 15 steps).
@@ -223,7 +223,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     // This grid may run beside the prepare kernel (programmatic dependent launch): it takes the length from the
     // caller's array with the same clamp, and waits for the prepare kernel (which clears the status record) only
     // where it is about to write that record, and at its end.
-    const int len = min(max(prm.cache_len_raw[b], 0), prm.max_len);
+    const int len = min(max(prm.cache_len[b], 0), prm.max_len);
     const int n_tiles = (len + T - 1) / T;
     const uint32_t* wrow = row_words(b, hk);
     // The splits of a row share its BYTES, not its tiles.  Split k of n takes the groups [bound(k C / n),
