@@ -1341,23 +1341,20 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
         if (prm.k_half_blocks) kernel = pick(std::true_type{});
     }
     if (ctas > 0x7fffffffLL) return static_cast<int>(cudaErrorInvalidConfiguration);
-    // Once per device and kernel instance: the shared-memory attribute, and a look at the registers.  The register split
-    // inside the kernel (setmaxnreg) assumes what the block is launched with; a build that gave the kernel fewer registers
-    // must not run (an increase beyond the block's allotment never returns).
-    constexpr int kMaxDev = 64;
-    static std::atomic<uint64_t> prepared[kMaxDev];      // bit per instance
+    // (set on every call: it belongs to the current context, and costs 0.07 us)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
+    if (e != cudaSuccess) return static_cast<int>(e);
+    // Once per kernel instance, a look at the registers it was built with (0.3 us).  The register split inside the kernel
+    // (setmaxnreg) assumes what the block is launched with; a build that gave the kernel fewer registers must not run (an
+    // increase beyond the block's allotment never returns).
+    static std::atomic<uint64_t> looked{0};      // bit per instance
     const uint64_t bit = 1ull << ((vl ? 1 : 0) + (dbg_on ? 2 : 0) + (otf ? 4 : 0) + (v_scale ? 8 : 0) + (prm.k_half_blocks ? 16 : 0) + (head_pair ? 32 : 0));
-    int device = 0;
-    if ((e = cudaGetDevice(&device)) != cudaSuccess) return static_cast<int>(e);
-    const bool known = device >= 0 && device < kMaxDev;
-    if (!known || !(prepared[device].load(std::memory_order_acquire) & bit)) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemAlloc);
-        if (e != cudaSuccess) return static_cast<int>(e);
+    if (!(looked.load(std::memory_order_acquire) & bit)) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, kernel);
         if (e != cudaSuccess) return static_cast<int>(e);
         if (fa.numRegs < (otf ? kLaunchRegsOtf : kLaunchRegs)) return TILEMIX_ERR_UNSUPPORTED;
-        if (known) prepared[device].fetch_or(bit, std::memory_order_release);
+        looked.fetch_or(bit, std::memory_order_release);
     }
     kernel<<<static_cast<unsigned>(ctas), otf ? kThreadsOtf : kThreads, C::kSmemAlloc, stream>>>(prm, tq, tk, tv, tq8, tk8);
     g_launch_count.fetch_add(1);

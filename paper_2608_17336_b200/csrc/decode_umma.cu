@@ -764,18 +764,8 @@ int encode_cache_map(EncodeTiledFn enc, CUtensorMap* tm, const void* base, int e
 template <int R>
 int launch_r(const DecodeParams& prm, const CUtensorMap& tk8, const CUtensorMap& tk16, cudaStream_t stream) {
     auto kernel = prm.k16 != nullptr ? decode_umma_kernel<R, true> : decode_umma_kernel<R, false>;
-    // the kernel's shared-memory attribute is set once per device and instance
-    constexpr int kMaxDev = 64;
-    static std::atomic<int> attr_set[kMaxDev][2];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);   // (of the current context)
     if (e != cudaSuccess) return static_cast<int>(e);
-    const int which = prm.k16 != nullptr ? 1 : 0;
-    if (dev < 0 || dev >= kMaxDev || attr_set[dev][which].load(std::memory_order_acquire) == 0) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return static_cast<int>(e);
-        if (dev >= 0 && dev < kMaxDev) attr_set[dev][which].store(1, std::memory_order_release);
-    }
     const dim3 grid = prm.balanced ? dim3(prm.n_ctas) : dim3(prm.n_splits, prm.Hk, prm.B);
     // programmatic dependent launch: this grid's set-up overlaps the tail of the prepare kernel
     cudaLaunchConfig_t cfg = {};

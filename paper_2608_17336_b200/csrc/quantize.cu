@@ -302,20 +302,12 @@ int rows_map(CUtensorMap* tm, const void* x, const int64_t stride[3], int B, int
 
 template <bool TILED, int W>
 int launch_stream_w(const QuantJobs& jobs, cudaStream_t stream, const CUtensorMap* maps) {
-    // SM count and the kernel's shared-memory attribute: asked for / set once per device
-    constexpr int kMaxDev = 64;
-    static std::atomic<int> sm_count[kMaxDev];
-    int dev = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // (set on every call: it belongs to the current context)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quantize_stream_kernel<TILED, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
     if (e != cudaSuccess) return static_cast<int>(e);
-    int sms = (dev >= 0 && dev < kMaxDev) ? sm_count[dev].load(std::memory_order_acquire) : 0;
-    if (sms == 0) {
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(quantize_stream_kernel<TILED, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-        if (e != cudaSuccess) return static_cast<int>(e);
-        if (dev >= 0 && dev < kMaxDev) sm_count[dev].store(sms, std::memory_order_release);
-    }
     const int grid = jobs.total < sms ? jobs.total : sms;
     quantize_stream_kernel<TILED, W><<<grid, kStreamThreads, kRingBytes, stream>>>(jobs, TILED ? maps[0] : CUtensorMap{},
                                                                                   TILED ? maps[1] : CUtensorMap{});
