@@ -936,7 +936,6 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
         const int quarter = warp & 3, t = (warp >> 2) & 1, sub = warp >> 3;
         const int m_t = t ? mB : mA;           // query tile
         const int rh = SUB ? quarter >> 1 : 0;                                    // row half of this warp's rows
-        const int r_t = SUB ? min(2 * m_t + rh, n_rows - 1) : m_t;                // their routing row (clamped: rows that do not exist)
         const int d_t = t ? dB : dA;           // step on the diagonal of the tile's first row
         if (t == 0 || hasB) {
             constexpr int TH = C::kTH;         // key columns per half step
@@ -1137,6 +1136,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             if (ok) {
                 // Finalise (Sec. 3.1): O = O~ / z in FP16; LSE = m + ln z.
                 ptx::tc_fence_after_sync();
+                bool row_valid[2];                     // rows beyond the sequence are not written
                 uint32_t o[SUB ? D / 32 : 1][16];
                 if constexpr (SUB) {
 #pragma unroll
@@ -1153,9 +1153,9 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     const float z_row = quad_sum(z[k]);
                     const int i_loc = m_t * T + rw[k];                            // row inside the sequence
                     const int64_t i_glob = static_cast<int64_t>(tok0) + i_loc;    // row on the token axis
-                    const bool row_valid = i_loc < len;
-                    z[k] = row_valid ? 1.f / z_row : 0.f;
-                    if (row_valid && cq == 0 && prm.lse != nullptr)
+                    row_valid[k] = i_loc < len;
+                    z[k] = 1.f / z_row;
+                    if (row_valid[k] && cq == 0 && prm.lse != nullptr)
                         prm.lse[(static_cast<int64_t>(b) * prm.Hq + hq + (t ? hp : 0)) * prm.L + i_glob] = (m_run[k] + log2f(z_row)) * kLn2;
                 }
                 // Two adjacent columns per lane and block of 8: a 4 x 4 transpose inside the quad gives every lane one
@@ -1186,7 +1186,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                             const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? w[i] : w[i + 2], 2);
                             if (upper) w[i] = got; else w[i + 2] = got;
                         }
-                        if (z[k] != 0.f)               // (0: a row beyond the sequence, not written)
+                        if (row_valid[k])
                             *reinterpret_cast<uint4*>(dst0 + rw[k] * prm.os[2] + c * 32) = make_uint4(w[0], w[1], w[2], w[3]);
                     }
                 }
@@ -1311,8 +1311,12 @@ int launch_impl(const Geometry& g, const void* q, const void* k, const void* v, 
         // same rows of two such heads: both take the same form of every key tile (adjacent rows of one head differ in 37 %
         // of the tiles at 75 % INT8, and then both copies have to be brought, 80 of the ring's 128 KB) and neither waits
         // for the other's last tile.  32 / 8 heads: 2048-token chunk of 24K 705 -> 645 us, packed batch of 16 prompts
-        // 515 -> 483, 8K 474 -> 450, the same on the fly 661 -> 633, 4 x 2K without INT8 groups 208 -> 202, 8 x 500 equal;
-        // 28 / 14 heads, 2 x 3000, 90 % INT8: 173 -> 175.
+        // 515 -> 483, 8K 474 -> 450, the same on the fly 661 -> 633, 4 x 2K without INT8 groups 208 -> 202, 8 x 500 equal.
+        // Taken at every even ratio: what decides is how often adjacent rows differ, which the host does not see.  Whole
+        // step, adjacent -> pairs, at 0 / 50 / 75 / 90 / 100 % INT8 groups: 32 / 16 heads, 16K 1804 -> 1847 / 2089 -> 1921 /
+        // 1927 -> 1829 / 1786 -> 1756 / 1704 -> 1724; 28 / 14, 2 x 3000 189 -> 198 / 200 -> 189 / 188 -> 183 / equal / 175 ->
+        // 177; 8 / 2, 16K 458 -> 470 / 474 -> 442 / 452 -> 427 / 441 -> 431 / 427 -> 431; 16 / 8, 4 x 2048 136 -> 130 / 142 ->
+        // 124 / 136 -> 124 / 130 -> 120 / 128 -> 118; d = 64: equal.
         head_pair = true;
         prm.single = 1;                            // (half as many pairs of heads, two CTAs per pair of tiles)
     }
