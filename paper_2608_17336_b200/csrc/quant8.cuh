@@ -32,8 +32,10 @@ __device__ __forceinline__ uint32_t umax2(uint32_t a, uint32_t b) { return __vma
 //  - x = amax / 2: the definition gives 64 if RN(x / delta) >= 63.5, else 63; r = RN(1 / delta) is moved by one unit in
 //    the last place where x * r falls on the other side of 63.5;
 //  - 127 divides the mantissa (then delta is exact; 8 of 1024 mantissas): `refine`, the quotient itself -- q0 = x * r,
-//    then q0 + (x - delta * q0) * r with the residual exact in one FMA -- before the rounding.
-// Both forms equal the definition for every binary16 amax and every |x| <= amax (all 5e8 pairs compared on the CPU).
+//    then q0 + (x - delta * q0) * r with the residual exact in one FMA (P. Markstein, "Computation of elementary functions
+//    on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990) -- before the rounding.
+// Both forms equal the definition for every binary16 amax and every |x| <= amax (tests/test_quant_codes.py compares the
+// arithmetic over all of them, tests/test_gpu_quant_exact.py the kernels next to the half-integers).
 // amax = inf or NaN: r = 0 or NaN, `refine` stays off.
 struct QuantScale {
     float delta, r;

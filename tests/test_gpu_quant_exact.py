@@ -10,7 +10,7 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("exponent", [0, 1, 15, 30])
+@pytest.mark.parametrize("exponent", [0, 1, 2, 8, 14, 15, 22, 29, 30])
 def test_codes_next_to_half_integers_for_every_maximum(exponent):
     from paper_2608_17336_b200 import binding as tm
     d, blk = 64, 64
