@@ -71,9 +71,6 @@ constexpr float kLn2 = 0.6931471805599453f;
 // P tops out at 2^-kMargin, 18 binades above the smallest FP16 subnormal, and a later score has to beat
 // everything before it by 2^(kMove + kMargin) to move m again.
 constexpr float kAccept = 8.0f, kMove = 4.0f, kMargin = 6.0f;
-// the INT8 route leaves the conversion bias to the scaling FMA while a * 1.5*2^23 <= kFoldLimit: the addend
-// m + a*1.5*2^23 is then below 2^13 and its rounding moves a score by at most 2^-12 (a relative 1.7e-4 in P)
-constexpr float kFoldLimit = 4096.0f;
 
 enum Role : int { kRoleSoftmaxA = 0, kRoleSoftmaxB = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQuant = 4 };
 enum Bar : int { kBarQ = 0, kBarRingFull = 1, kBarRingEmpty = 2, kBarS = 3, kBarP = 4, kBarO = 5, kBarDrain = 6, kBarPV = 7,
@@ -990,25 +987,13 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 uint32_t p[2 * NB];
                 ptx::tmem_wait_ld_dep(s);     // ties the registers to the wait: no use of them moves above it
                 if (!redo) {
+                    const float addend[2] = {-m_run[0], -m_run[1]};
                     if (!int8_route) {
-                        const float addend[2] = {-m_run[0], -m_run[1]};
-                        softmax_step_fast<NB, kFp32, VS>(s, a, addend, p, sum, dv);
-                    } else if constexpr (KH) {
-                        if (fmaxf(a, a_hi) * kInt8Bias <= kFoldLimit) {
-                            const float addend[2] = {-__fmaf_rn(a, kInt8Bias, m_run[0]), -__fmaf_rn(a, kInt8Bias, m_run[1])};
-                            const float addend_hi[2] = {-__fmaf_rn(a_hi, kInt8Bias, m_run[0]), -__fmaf_rn(a_hi, kInt8Bias, m_run[1])};
-                            softmax_step_fast2<NB, kInt8Folded, VS>(s, a, addend, a_hi, addend_hi, p, sum, dv);
-                        } else {
-                            const float addend[2] = {-m_run[0], -m_run[1]};
-                            softmax_step_fast2<NB, kInt8Exact, VS>(s, a, addend, a_hi, addend, p, sum, dv);
-                        }
-                    } else if (a * kInt8Bias <= kFoldLimit) {
-                        // one explicit FMA: every instantiation of the kernel rounds the addend the same way
-                        const float addend[2] = {-__fmaf_rn(a, kInt8Bias, m_run[0]), -__fmaf_rn(a, kInt8Bias, m_run[1])};
-                        softmax_step_fast<NB, kInt8Folded, VS>(s, a, addend, p, sum, dv);
+                        if constexpr (KH) softmax_step_fast2<NB, false, VS>(s, a, a_hi, addend, p, sum, dv);
+                        else softmax_step_fast<NB, false, VS>(s, a, addend, p, sum, dv);
                     } else {
-                        const float addend[2] = {-m_run[0], -m_run[1]};
-                        softmax_step_fast<NB, kInt8Exact, VS>(s, a, addend, p, sum, dv);
+                        if constexpr (KH) softmax_step_fast2<NB, true, VS>(s, a, a_hi, addend, p, sum, dv);
+                        else softmax_step_fast<NB, true, VS>(s, a, addend, p, sum, dv);
                     }
                     // The store of P goes out before the vote, so that the vote's latency hides behind it; a rejected
                     // step stores again below, after this store has been waited for.

@@ -42,32 +42,23 @@ __device__ __forceinline__ float quad_sum(float v) {
     return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
-// How the raw accumulators of a step become floats: FP32 scores as they are; INT32 scores by the bias trick --
-// bits(1.5*2^23) + i is the float 1.5*2^23 + i for |i| < 2^22 (here |i| <= 127*127*D) -- either with the bias
-// removed by an exact subtraction before the scaling (kInt8Exact), or left in and cancelled by the addend of the
-// scaling FMA, a*(1.5*2^23 + i) - (m + a*1.5*2^23) (kInt8Folded: one instruction less per pair; the addend is
-// rounded once per step, so the caller uses it only while that rounding is negligible).
-enum ScoreKind : int { kFp32 = 0, kInt8Exact = 1, kInt8Folded = 2 };
-constexpr float kInt8Bias = 12582912.f;   // 1.5 * 2^23
-
 // Blocks I0 .. I1 - 1 of a step of NB, see softmax_step_fast; acc = packed partial row sums.
-template <int I0, int I1, int NB, int KIND, bool VS>
+// INT32 scores become floats with the conversion instruction: 2 clk per warp instruction and scheduler, and none of the
+// special-function unit's time (ex2 alone 8.02 clk, with a conversion beside each 8.00).  The bias trick it replaced
+// (1.5 * 2^23 + i as bits, the bias taken back by the addend of the scaling FMA while its rounding was negligible, else by
+// a subtraction) took as many instructions in its folded form and one more per pair in the other, which inputs with large
+// block scales fell into, and a second copy of this code: 8K with outlier channels 632 -> 621 us, others 0 to -0.8 %.
+template <int I0, int I1, int NB, bool INT8, bool VS>
 __device__ __forceinline__ void softmax_blocks(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2],
                                                uint32_t (&p)[2 * NB], float2 (&acc)[2], float dv) {
     const float2 a2 = make_float2(a, a);
-    const float2 unbias = make_float2(-kInt8Bias, -kInt8Bias);
 #pragma unroll
     for (int i = I0; i < I1; ++i) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const uint32_t r0 = s[4 * i + 2 * k], r1 = s[4 * i + 2 * k + 1];
-            float2 x;
-            if (KIND == kFp32) {
-                x = make_float2(__uint_as_float(r0), __uint_as_float(r1));
-            } else {
-                x = make_float2(__uint_as_float(r0 + 0x4B400000u), __uint_as_float(r1 + 0x4B400000u));
-                if (KIND == kInt8Exact) x = __fadd2_rn(x, unbias);
-            }
+            const float2 x = INT8 ? make_float2(__int2float_rn(static_cast<int>(r0)), __int2float_rn(static_cast<int>(r1)))
+                                  : make_float2(__uint_as_float(r0), __uint_as_float(r1));
             const float2 t2 = __ffma2_rn(x, a2, make_float2(addend[k], addend[k]));
             const float2 e = make_float2(fast_exp2(t2.x), fast_exp2(t2.y));
             acc[k] = __fadd2_rn(acc[k], e);
@@ -82,27 +73,26 @@ __device__ __forceinline__ void softmax_blocks(const uint32_t (&s)[4 * NB], floa
 }
 
 // One interior step (NB blocks of 8 key columns, no causal mask) in one pass with the current running
-// maxima: raw accumulators s -> P = 2^(a*raw - m) rounded to FP16 (p[2i + k] = the pair of row k in block
-// i) and this thread's part of the FP32 row sums.  addend[k] = -m_k (kFp32, kInt8Exact) or -(m_k + a*1.5*2^23)
-// (kInt8Folded).  VS: the probabilities are multiplied by `dv` (the block scale of an INT8 value cache, App. C:
-// folded into the probability tile) before they are rounded to FP16; the row sums are of the unscaled values.
-template <int NB, int KIND, bool VS = false>
+// maxima: raw accumulators s (INT32 on the INT8 route, else FP32) -> P = 2^(a*raw - m) rounded to FP16 (p[2i + k] = the
+// pair of row k in block i) and this thread's part of the FP32 row sums.  addend[k] = -m_k.  VS: the probabilities are
+// multiplied by `dv` (the block scale of an INT8 value cache, App. C: folded into the probability tile) before they are
+// rounded to FP16; the row sums are of the unscaled values.
+template <int NB, bool INT8, bool VS = false>
 __device__ __forceinline__ void softmax_step_fast(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2],
                                                   uint32_t (&p)[2 * NB], float (&sum)[2], float dv = 1.f) {
     float2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-    softmax_blocks<0, NB, NB, KIND, VS>(s, a, addend, p, acc, dv);
+    softmax_blocks<0, NB, NB, INT8, VS>(s, a, addend, p, acc, dv);
     sum[0] = acc[0].x + acc[0].y;
     sum[1] = acc[1].x + acc[1].y;
 }
 
-// The same with one scaling factor (and addend) for the first and one for the second half of the columns.
-template <int NB, int KIND, bool VS = false>
-__device__ __forceinline__ void softmax_step_fast2(const uint32_t (&s)[4 * NB], float a, const float (&addend)[2], float a_hi,
-                                                   const float (&addend_hi)[2], uint32_t (&p)[2 * NB], float (&sum)[2],
-                                                   float dv = 1.f) {
+// The same with one scaling factor for the first and one for the second half of the columns.
+template <int NB, bool INT8, bool VS = false>
+__device__ __forceinline__ void softmax_step_fast2(const uint32_t (&s)[4 * NB], float a, float a_hi, const float (&addend)[2],
+                                                   uint32_t (&p)[2 * NB], float (&sum)[2], float dv = 1.f) {
     float2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-    softmax_blocks<0, NB / 2, NB, KIND, VS>(s, a, addend, p, acc, dv);
-    softmax_blocks<NB / 2, NB, NB, KIND, VS>(s, a_hi, addend_hi, p, acc, dv);
+    softmax_blocks<0, NB / 2, NB, INT8, VS>(s, a, addend, p, acc, dv);
+    softmax_blocks<NB / 2, NB, NB, INT8, VS>(s, a_hi, addend, p, acc, dv);
     sum[0] = acc[0].x + acc[0].y;
     sum[1] = acc[1].x + acc[1].y;
 }
