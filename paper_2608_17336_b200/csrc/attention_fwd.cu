@@ -62,15 +62,18 @@ constexpr int kWorkspaceClearBytes = 4096;  // status record
 constexpr int kMaxTiles = 2048;           // key tiles per row the shared-memory schedule table holds
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-// Lazy running maximum.  P = 2^(score - m) is handed to the tensor pipe in FP16 (largest finite value just
-// below 2^16), z and O are FP32, so m may lag the true row maximum.  An interior step is done in one pass with
-// the current m and is accepted when this thread's part of each row sum stays below 2^kAccept (no probability
-// of the step can then exceed 2^kAccept).  Otherwise the step is redone from the accumulators in the generic
-// two-pass form, which moves m to kMargin above the step's maximum whenever that maximum is more than kMove above
-// m (a rejected step always is: 2^kAccept spread over at most 16 values) and rescales z and O.  After a move
-// P tops out at 2^-kMargin, 18 binades above the smallest FP16 subnormal, and a later score has to beat
-// everything before it by 2^(kMove + kMargin) to move m again.
-constexpr float kAccept = 8.0f, kMove = 4.0f, kMargin = 6.0f;
+// Lazy running maximum.  P = 2^(score - m) is handed to the tensor pipe in FP16 (largest finite value 65504), z and O
+// are FP32, so m may lag the true row maximum.  An interior step is done in one pass with the current m and is accepted
+// when this thread's part of each row sum stays below kAccept (no probability of the step can then exceed it).  Otherwise
+// the step is redone from the accumulators in the generic two-pass form, which moves m to kMargin above the step's maximum
+// whenever that maximum is more than kMove above m (a rejected step always is: kAccept spread over at most 16 values) and
+// rescales z and O.  After a move P tops out at 2^-kMargin, 18 binades above the smallest FP16 subnormal, and a later
+// score has to beat everything before it by a factor of kAccept * 2^kMargin to move m again.
+// A redone step costs its tile a second pass and a wait for the PV in flight, and with 128 rows that move m on their own
+// account it is hardly ever one row's affair: kAccept is half of what FP16 holds, not less (at 2^8, 32 heads x 8K with
+// outlier channels took 628 us in place of 590; maps and inputs whose m rarely moves take the same time).
+// An INT8 value cache multiplies P by its block's scale before it is rounded, up to 65504 / 127: kAcceptScaled.
+constexpr float kAccept = 32768.f, kAcceptScaled = 256.f, kMove = 4.0f, kMargin = 6.0f;
 
 enum Role : int { kRoleSoftmaxA = 0, kRoleSoftmaxB = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQuant = 4 };
 enum Bar : int { kBarQ = 0, kBarRingFull = 1, kBarRingEmpty = 2, kBarS = 3, kBarP = 4, kBarO = 5, kBarDrain = 6, kBarPV = 7,
@@ -999,7 +1002,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     // step stores again below, after this store has been waited for.
                     ptx::tmem_st16x128_x8(t_sh, p);
                     stored = true;
-                    redo = __any_sync(0xffffffffu, !(sum[0] <= exp2f(kAccept) && sum[1] <= exp2f(kAccept)));   // also true for a NaN
+                    constexpr float kMost = VS ? kAcceptScaled : kAccept;
+                    redo = __any_sync(0xffffffffu, !(sum[0] <= kMost && sum[1] <= kMost));   // also true for a NaN
                 }
                 if (redo) {
                     // Generic two-pass form: the very first step, the diagonal tile, steps that move the maximum, and
