@@ -111,10 +111,10 @@ struct Cfg {
     static constexpr int kOffBars = kOffRing + kRing * kChunk;
     static constexpr int kTH = T / 2;                 // key columns per half step
     static constexpr int kNumBars = 2 + 2 * kRing + 4 + 4 + 2 + 2 + 1 + kBundles + 2;
-    static constexpr int kOffMisc = kOffBars + kNumBars * 8;       // tmem base, abort flag; on-chip scales
+    static constexpr int kOffMisc = kOffBars + kNumBars * 8;       // tmem base, abort flag; on-chip scales; work item
     // ring of the softmax warps' scaling factors: kScSlots key tiles of kScStride floats (see the scale warp)
     static constexpr int kScSlots = 16, kScStride = kSub ? 32 : 8;
-    static constexpr int kOffSc = kOffMisc + 64;
+    static constexpr int kOffSc = kOffMisc + 96;
     static constexpr int kOffWords = kOffSc + kScSlots * kScStride * 4;
     static constexpr int kSmemBytes = kOffWords + kMaxTiles / 2;   // 4-bit schedule entries
     static constexpr int kSmemAlloc = kSmemBytes + 1024;           // slack to align the base
@@ -314,6 +314,10 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
     auto bar_raw = [&](int i) { return bar0 + 8u * (15 + 2 * kRing + i); };
     auto bar_q8 = [&](int t) { return bar0 + 8u * (15 + 2 * kRing + kBundles + t); };
     uint32_t* misc = reinterpret_cast<uint32_t*>(smem + C::kOffMisc);   // [0] tmem base, [1] abort
+    // The work item once more, for the epilogue: what the softmax warps would carry through their loop costs them registers
+    // there, and spilled ones are reloaded step by step (mixed 32K 6565 -> 6510 us, 128K 26.33 -> 25.8 ms, 2K chunk of 24K
+    // 647 -> 638, 8K 590 -> 583, 8 x 4K 1192 -> 1186).
+    volatile int* item_s = reinterpret_cast<volatile int*>(misc + 16);
     // Scaling factors of the softmax steps.  Key tile j's are in slot j % kScSlots, written before bundle j's "landed"
     // barrier completes; by then bundle j - 2 kBundles has been consumed, so every softmax warp is past key tile
     // j - 2 kBundles - 1 and the slot is free.  Factor of (half h, tile t, row half r, 32-key half q): index
@@ -340,6 +344,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             ptx::mbar_init(bar_q(1), 1);
             ptx::mbar_init(bar_full(0), OTF ? 1 + kQuantWarps : 2);
             misc[1] = 0;
+            item_s[0] = b; item_s[1] = hq; item_s[2] = tok0; item_s[3] = len; item_s[4] = mA; item_s[5] = mB;
         } else if (lane == 1) {      // (bar_full(0): lane 0)
         } else if (lane <= 3 * kBundles) {
             // on-the-fly mode: one more arrival per quantiser warp on "landed" (after it made its rows of the bundle's
@@ -1125,6 +1130,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
             if (ok) {
                 // Finalise (Sec. 3.1): O = O~ / z in FP16; LSE = m + ln z.
                 ptx::tc_fence_after_sync();
+                const int b = item_s[0], hq = item_s[1], tok0 = item_s[2], len = item_s[3], m_t = item_s[4 + t];
                 bool row_valid[2];                     // rows beyond the sequence are not written
                 uint32_t o[SUB ? D / 32 : 1][16];
                 if constexpr (SUB) {
