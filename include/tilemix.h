@@ -314,7 +314,7 @@ typedef struct tilemix_decode {
     float softmax_scale;   /* <= 0 means 1/sqrt(head_dim)                                   */
 } tilemix_decode_t;
 
-/* Bytes of `workspace` for tilemix_decode_int8kv: the status record, a reserved area of four bytes per sequence
+/* Bytes of `workspace` for tilemix_decode_int8kv: the status record, an area of four bytes per sequence for counters
  * and the partial results of the splits (0 on an invalid problem). */
 size_t tilemix_decode_workspace_size(const tilemix_decode_t* p);
 /*   q_f16      FP16 [B, Hq, d]
@@ -330,8 +330,9 @@ size_t tilemix_decode_workspace_size(const tilemix_decode_t* p);
  *   out_f16    FP16 [B, Hq, d];  lse nullable FP32 [B, Hq]
  *   q_i8_out / q_scale_out  nullable INT8 [B, Hq, d] / FP32 [B, Hq]: the quantised query the
  *              kernel used (for checking)
- * Three kernels are enqueued on `stream` (one that clears the status record, the step over the splits, the merge;
- * the last two are programmatic dependent launches, so that their set-up overlaps the kernel before them).  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
+ * Two or three kernels are enqueued on `stream`: one that clears the status record and the rows' counters; the step, a
+ * programmatic dependent launch whose set-up overlaps it; and, where the CTAs of the step do not start together, a merge of
+ * the splits, programmatic dependent as well (elsewhere the last CTA of a row merges them).  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
  * kernel itself found (a bounded wait that ran out, or the missing FP16 cache above). */
 int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const void* k_f16,
                           const int8_t* k_i8, const float* k_scale, const int8_t* v_i8,

@@ -18,8 +18,6 @@ namespace tilemix {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLn2 = 0.6931471805599453f;
-
 
 // Keys per kernel tile.  Head dimension 64: 128, i.e. one routing tile of 128 keys or two of 64 (each of the eight warps
 // has a 16-key step of its own).  Head dimension 128 (64-key routing tiles): 64, two warps per step with half of the
@@ -498,65 +496,35 @@ decode_kernel(const DecodeParams prm) {
         prm.o_part[row * D + e] = o;
         if (e == 0) { prm.m_part[row] = m; prm.z_part[row] = z; }
     }
+    if (prm.fused) merge_if_last<D, R>(prm, b, hk, prm.n_splits, prm.n_splits);
 }
 
-// Merge of the splits: m = max m_s, z = sum z_s 2^(m_s - m), O = sum O~_s 2^(m_s - m) / z.  One block per query head,
-// one thread per output element.  The parts are taken 32 at a time: lane s of every warp loads (m_s, z_s) and the
-// weights are shared by shuffles, so that the loads of O~_s depend on one round trip only and are in flight
-// together (a part that nobody wrote has m_s = -inf, weight 0, and is not loaded).
+// Merge as a kernel of its own (grids of several waves, see tilemix_decode_int8kv): one block per query head, one thread per
+// output column.
 template <int D>
 __global__ void __launch_bounds__(D)
-decode_merge_kernel(const float* __restrict__ o_part, const float* __restrict__ m_part,
-                    const float* __restrict__ z_part, int n_splits, __half* __restrict__ out,
-                    float* __restrict__ lse) {
+decode_merge_kernel(const DecodeParams prm) {
     ptx::griddep_wait();   // (when launched as a programmatic dependent of the step kernel)
-    const int64_t row = blockIdx.x;
-    const int e = threadIdx.x, lane = e & 31;
-    float m = -INFINITY, z = 0.f, o = 0.f;
-    for (int s0 = 0; s0 < n_splits; s0 += 32) {
-        const int s = s0 + lane;
-        const float ms = s < n_splits ? m_part[row * n_splits + s] : -INFINITY;
-        const float zs = s < n_splits ? z_part[row * n_splits + s] : 0.f;
-        float mc = ms;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, d));
-        const float m_new = fmaxf(m, mc);
-        if (m_new == -INFINITY) continue;                    // (the same in every lane)
-        const float back = m == -INFINITY ? 0.f : exp2f(m - m_new);
-        const float w = ms == -INFINITY ? 0.f : exp2f(ms - m_new);
-        const float zw = ms == -INFINITY ? 0.f : zs * w;
-        z *= back; o *= back; m = m_new;
-        const int cnt = min(32, n_splits - s0);
-        const float* src = o_part + (row * n_splits + s0) * D + e;
-#pragma unroll 8
-        for (int i = 0; i < cnt; ++i) {
-            const float wi = __shfl_sync(0xffffffffu, w, i);
-            z += __shfl_sync(0xffffffffu, zw, i);
-            if (wi != 0.f) o += src[static_cast<int64_t>(i) * D] * wi;
-        }
-    }
-    out[row * D + e] = __float2half_rn(z > 0.f ? o / z : 0.f);
-    if (e == 0 && lse != nullptr) lse[row] = z > 0.f ? (m + log2f(z)) * kLn2 : -INFINITY;
+    merge_column<D>(prm, blockIdx.x, prm.n_parts, threadIdx.x);
 }
 
 // Step and merge overlap the tail of the kernel before them (programmatic dependent launch).
 template <int D>
-int launch_merge(const DecodeParams& prm, int n_splits, __half* out, float* lse, cudaStream_t stream) {
+int launch_merge(const DecodeParams& prm, cudaStream_t stream) {
+    if (prm.fused) return TILEMIX_OK;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(prm.B * prm.Hq); cfg.blockDim = dim3(D); cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_merge_kernel<D>, static_cast<const float*>(prm.o_part),
-                                             static_cast<const float*>(prm.m_part), static_cast<const float*>(prm.z_part),
-                                             n_splits, out, lse);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, decode_merge_kernel<D>, prm);
     g_launch_count.fetch_add(1);
     return static_cast<int>(e);
 }
 
 template <int D, int R, int RT>
-int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t stream) {
+int launch_cfg(const DecodeParams& prm, cudaStream_t stream) {
     // no FP16 key cache: the instance whose ring holds INT8 keys only
     auto kernel = prm.k16 != nullptr ? decode_kernel<D, R, RT, true> : decode_kernel<D, R, RT, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
@@ -571,16 +539,16 @@ int launch_cfg(const DecodeParams& prm, __half* out, float* lse, cudaStream_t st
     e = cudaLaunchKernelEx(&cfg, kernel, prm);
     g_launch_count.fetch_add(1);
     if (e != cudaSuccess) return static_cast<int>(e);
-    return launch_merge<D>(prm, prm.n_splits, out, lse, stream);
+    return launch_merge<D>(prm, stream);
 }
 
 template <int D, int RT>
-int launch_r(int R, const DecodeParams& prm, __half* out, float* lse, cudaStream_t stream) {
+int launch_r(int R, const DecodeParams& prm, cudaStream_t stream) {
     switch (R) {
-        case 1: return launch_cfg<D, 1, RT>(prm, out, lse, stream);
-        case 2: return launch_cfg<D, 2, RT>(prm, out, lse, stream);
-        case 4: return launch_cfg<D, 4, RT>(prm, out, lse, stream);
-        case 8: return launch_cfg<D, 8, RT>(prm, out, lse, stream);
+        case 1: return launch_cfg<D, 1, RT>(prm, stream);
+        case 2: return launch_cfg<D, 2, RT>(prm, stream);
+        case 4: return launch_cfg<D, 4, RT>(prm, stream);
+        case 8: return launch_cfg<D, 8, RT>(prm, stream);
         default: return TILEMIX_ERR_UNSUPPORTED;
     }
 }
@@ -589,14 +557,14 @@ constexpr size_t kDecodeStatusBytes = 256;   // status record of the bounded wai
 constexpr int kDecodeWave = 148;             // CTAs of one wave of the tcgen05 form (one per SM)
 constexpr int kDecodeBalanceRows = 160;      // rows of a batch whose splits that kernel can balance
 
-// Before the step: clears the status record.  (The cache lengths live on the device, so the host cannot check them: the
-// step clamps each to [0, max_len] as it reads it.)
-__global__ void decode_prepare_kernel(int* status) {
-    ptx::griddep_launch_dependents();   // the step kernel may start meanwhile; it waits before it writes the record or ends
-    if (threadIdx.x < 4) status[threadIdx.x] = 0;
+// Before the step: clears the status record and the rows' counters behind it.  (The cache lengths live on the device, so the
+// host cannot check them: the step clamps each to [0, max_len] as it reads it.)
+__global__ void decode_prepare_kernel(int* status, int n) {
+    ptx::griddep_launch_dependents();   // the step kernel may start meanwhile; it waits before it uses either or ends
+    for (int i = threadIdx.x; i < n; i += blockDim.x) status[i] = 0;
 }
 
-// Reserved behind the status record (it held a copy of the lengths): the size of a workspace stays what it was.
+// Behind the status record (it held a copy of the lengths): room for counters.  The size of a workspace stays what it was.
 size_t decode_len_bytes(int B) { return (static_cast<size_t>(B) * sizeof(int32_t) + 255) / 256 * 256; }
 
 struct DecodeGeometry {
@@ -728,20 +696,31 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     prm.q8_out = q_i8_out; prm.qs_out = q_scale_out;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int R = p->heads_q / p->heads_kv;
-    __half* out = static_cast<__half*>(out_f16);
-    decode_prepare_kernel<<<1, 32, 0, s>>>(prm.status);
+    prm.out = static_cast<__half*>(out_f16);
+    prm.lse = lse;
+    // The step merges a row's splits itself where its CTAs start together (one wave, or the shared-out form): a launch and
+    // the end of the grid less; us with a merge kernel and so: 1 sequence, 32 / 8 heads of 128, 4096 keys 23.4 / 19.3, 64K
+    // keys 54 / 48; heads of 64, 8192 keys 27.4 / 17.3; 16 ragged sequences shared out 76.5 / 74.6; 8 x 32K equal.  In a
+    // grid of several waves the merge at the end of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000,
+    // 32 KV heads 137 / 146.  Every row needs a counter behind the status record (there are 248 with up to 64 sequences).
+    const int words = static_cast<int>((kDecodeStatusBytes + decode_len_bytes(p->batch)) / 4) - 4, n_words = (prm.n_rows + 1) / 2;
+    const bool umma = p->head_dim == 128 && p->tile_n == 128;
+    const int64_t ctas = static_cast<int64_t>(g.n_splits) * prm.n_rows, wave = umma ? kDecodeWave : 2 * kDecodeWave;
+    prm.fused = n_words <= words && g.n_splits <= 0xffff && (g.balanced || (g.n_splits > 1 && ctas <= wave)) ? 1 : 0;
+    prm.arrived = reinterpret_cast<uint32_t*>(prm.status) + 4;
+    decode_prepare_kernel<<<1, 128, 0, s>>>(prm.status, prm.fused ? 4 + n_words : 4);
     g_launch_count.fetch_add(1);
     cudaError_t pe = cudaGetLastError();
     if (pe != cudaSuccess) return static_cast<int>(pe);
-    if (p->head_dim == 128 && p->tile_n == 128) {
+    if (umma) {
         // the tcgen05 form of the step (decode_umma.cu), then the same merge
         rc = launch_decode_umma(R, prm, s);
         if (rc) return rc;
-        return launch_merge<128>(prm, g.n_parts, out, lse, s);
+        return launch_merge<128>(prm, s);
     }
-    if (p->head_dim == 128 && p->tile_n == 64) return launch_r<128, 64>(R, prm, out, lse, s);
-    if (p->head_dim == 64 && p->tile_n == 128) return launch_r<64, 128>(R, prm, out, lse, s);
-    if (p->head_dim == 64 && p->tile_n == 64) return launch_r<64, 64>(R, prm, out, lse, s);
+    if (p->head_dim == 128 && p->tile_n == 64) return launch_r<128, 64>(R, prm, s);
+    if (p->head_dim == 64 && p->tile_n == 128) return launch_r<64, 128>(R, prm, s);
+    if (p->head_dim == 64 && p->tile_n == 64) return launch_r<64, 64>(R, prm, s);
     return TILEMIX_ERR_UNSUPPORTED;
 }
 

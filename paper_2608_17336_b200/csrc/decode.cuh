@@ -4,6 +4,7 @@
 
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace tilemix {
@@ -29,10 +30,73 @@ struct DecodeParams {
     float* z_part;
     int8_t* q8_out;
     float* qs_out;
+    __half* out;     // [B, Hq, D]
+    float* lse;      // nullable [B, Hq]
+    // 16 bits per (sequence, KV head) row, 0 before the step: CTAs of the row that have written their partial results.  The
+    // last one merges them.
+    uint32_t* arrived;
+    int fused;       // 1: merged by the step, 0: by a kernel of its own
     int* status;     // 4 ints at the start of the workspace (same record as the attention kernel's)
     unsigned long long wait_limit_ns;   // limit of the bounded waits
     int test_drop_tile;                 // testing aid: the producer leaves out the copies of this tile of every split (-1: none)
 };
+
+// Merge of partial results: m = max m_s, z = sum z_s 2^(m_s - m), O = sum O~_s 2^(m_s - m) / z for the query head `row` of
+// [B, Hq] and output column e; a whole warp with consecutive columns.  The parts are taken 32 at a time: lane s loads
+// (m_s, z_s) and the weights are shared by shuffles, so that the loads of O~_s depend on one round trip only and are in
+// flight together (a part that nobody wrote has m_s = -inf, weight 0, and is not loaded).
+template <int D>
+__device__ __forceinline__ void merge_column(const DecodeParams& prm, int64_t row, int n_parts, int e) {
+    constexpr float kLn2f = 0.6931471805599453f;
+    const int lane = threadIdx.x & 31;
+    const int64_t first = row * prm.n_parts;
+    float m = -INFINITY, z = 0.f, o = 0.f;
+    for (int s0 = 0; s0 < n_parts; s0 += 32) {
+        const int s = s0 + lane;
+        const float ms = s < n_parts ? __ldcg(prm.m_part + first + s) : -INFINITY;
+        const float zs = s < n_parts ? __ldcg(prm.z_part + first + s) : 0.f;
+        float mc = ms;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, d));
+        const float m_new = fmaxf(m, mc);
+        if (m_new == -INFINITY) continue;                    // (the same in every lane)
+        const float back = m == -INFINITY ? 0.f : exp2f(m - m_new);
+        const float w = ms == -INFINITY ? 0.f : exp2f(ms - m_new);
+        const float zw = ms == -INFINITY ? 0.f : zs * w;
+        z *= back; o *= back; m = m_new;
+        const int cnt = min(32, n_parts - s0);
+        const float* src = prm.o_part + (first + s0) * D + e;
+#pragma unroll 8
+        for (int i = 0; i < cnt; ++i) {
+            const float wi = __shfl_sync(0xffffffffu, w, i);
+            z += __shfl_sync(0xffffffffu, zw, i);
+            if (wi != 0.f) o += __ldcg(src + static_cast<int64_t>(i) * D) * wi;
+        }
+    }
+    prm.out[row * D + e] = __float2half_rn(z > 0.f ? o / z : 0.f);
+    if (e == 0 && prm.lse != nullptr) prm.lse[row] = z > 0.f ? (m + log2f(z)) * kLn2f : -INFINITY;
+}
+
+// At the end of a step's CTA, by all its threads, when the partial results that it owes have been stored: the last CTA of
+// row (b, hk) -- `ctas` of them -- merges the n_parts parts of its R query heads.
+template <int D, int R>
+__device__ __forceinline__ void merge_if_last(const DecodeParams& prm, int b, int hk, int ctas, int n_parts) {
+    __shared__ int last_s;
+    if (ctas > 1) __threadfence();        // this thread's partial results, before the arrival
+    __syncthreads();
+    if (ctas > 1) {
+        if (threadIdx.x == 0) {
+            const int row = b * prm.Hk + hk;
+            const uint32_t before = atomicAdd(prm.arrived + (row >> 1), 1u << (16 * (row & 1)));
+            last_s = static_cast<int>((before >> (16 * (row & 1))) & 0xffffu) == ctas - 1;
+        }
+        __syncthreads();
+        if (!last_s) return;
+        __threadfence();
+    }
+    for (int i = threadIdx.x; i < R * D; i += blockDim.x)
+        merge_column<D>(prm, static_cast<int64_t>(b) * prm.Hq + hk * R + i / D, n_parts, i % D);
+}
 
 // The tcgen05 form of the step for head_dim 128, tile_n 128 (R = Hq / Hk in {1, 2, 4, 8}): enqueues the kernel
 // that writes (m, z, O~) of every split to the workspace; the caller launches the merge.  Returns a cudaError_t

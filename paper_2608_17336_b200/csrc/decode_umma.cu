@@ -259,9 +259,9 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     // shared memory (to_smem), and -- from the one split of the row that starts at its first group -- the quantised
     // row and its scale to the caller's buffers.
     const bool q_writer = g0 == 0 && (g1 > 0 || split + 1 == row_splits);
-    // parts of the row that no split writes (balanced form: the row has fewer splits than the workspace has room
+    // (merged by a kernel of its own) parts of the row that no split writes (balanced form: the row has fewer splits than the workspace has room
     // for): marked empty for the merge by the row's first split
-    if (split == 0)
+    if (split == 0 && !prm.fused)
         for (int idx = tid; idx < R * (n_parts - kStreams * row_splits); idx += kThreads) {
             const int r = idx / (n_parts - kStreams * row_splits), part = kStreams * row_splits + idx % (n_parts - kStreams * row_splits);
             prm.m_part[(static_cast<int64_t>(b) * prm.Hq + hk * R + r) * n_parts + part] = -INFINITY;
@@ -308,6 +308,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         }
         if (q_writer && warp < R) prep_query_row(warp, false);   // (a row without keys still reports its quantised query)
         leave();
+        if (prm.fused) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
         return;
     }
 
@@ -740,6 +741,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, kTmemCols);
     }
+    if (prm.fused && !*abort_flag) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
