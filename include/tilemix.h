@@ -331,8 +331,8 @@ size_t tilemix_decode_workspace_size(const tilemix_decode_t* p);
  *   q_i8_out / q_scale_out  nullable INT8 [B, Hq, d] / FP32 [B, Hq]: the quantised query the
  *              kernel used (for checking)
  * Two or three kernels are enqueued on `stream`: one that clears the status record and the rows' counters; the step, a
- * programmatic dependent launch whose set-up overlaps it; and, where the CTAs of the step do not start together, a merge of
- * the splits, programmatic dependent as well (elsewhere the last CTA of a row merges them).  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
+ * programmatic dependent launch whose set-up overlaps it; and, where the step does not merge a row's splits itself, a merge
+ * kernel, programmatic dependent as well.  Errors as for the other entry points; tilemix_read_status on the workspace reports what the
  * kernel itself found (a bounded wait that ran out, or the missing FP16 cache above). */
 int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const void* k_f16,
                           const int8_t* k_i8, const float* k_scale, const int8_t* v_i8,

@@ -18,6 +18,7 @@ namespace tilemix {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kLn2 = 0.6931471805599453f;
 
 // Keys per kernel tile.  Head dimension 64: 128, i.e. one routing tile of 128 keys or two of 64 (each of the eight warps
 // has a 16-key step of its own).  Head dimension 128 (64-key routing tiles): 64, two warps per step with half of the
@@ -492,11 +493,16 @@ decode_kernel(const DecodeParams prm) {
                 z += red[w][r][D + 1] * wgt;
             }
         }
-        const int64_t row = (static_cast<int64_t>(b) * prm.Hq + hk * R + r) * prm.n_splits + split;
-        prm.o_part[row * D + e] = o;
-        if (e == 0) { prm.m_part[row] = m; prm.z_part[row] = z; }
+        const int64_t head = static_cast<int64_t>(b) * prm.Hq + hk * R + r, part = head * prm.n_splits + split;
+        if (prm.n_splits == 1) {
+            prm.out[head * D + e] = __float2half_rn(z > 0.f ? o / z : 0.f);
+            if (e == 0 && prm.lse != nullptr) prm.lse[head] = z > 0.f ? (m + log2f(z)) * kLn2 : -INFINITY;
+        } else {
+            prm.o_part[part * D + e] = o;
+            if (e == 0) { prm.m_part[part] = m; prm.z_part[part] = z; }
+        }
     }
-    if (prm.fused) merge_if_last<D, R>(prm, b, hk, prm.n_splits, prm.n_splits);
+    if (prm.fused && prm.n_splits > 1) merge_if_last<D, R>(prm, b, hk, prm.n_splits, prm.n_splits);
 }
 
 // Merge as a kernel of its own (grids of several waves, see tilemix_decode_int8kv): one block per query head, one thread per
@@ -698,17 +704,23 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     const int R = p->heads_q / p->heads_kv;
     prm.out = static_cast<__half*>(out_f16);
     prm.lse = lse;
-    // The step merges a row's splits itself where its CTAs start together (one wave, or the shared-out form): a launch and
-    // the end of the grid less; us with a merge kernel and so: 1 sequence, 32 / 8 heads of 128, 4096 keys 23.4 / 19.3, 64K
-    // keys 54 / 48; heads of 64, 8192 keys 27.4 / 17.3; 16 ragged sequences shared out 76.5 / 74.6; 8 x 32K equal.  In a
-    // grid of several waves the merge at the end of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000,
-    // 32 KV heads 137 / 146.  Every row needs a counter behind the status record (there are 248 with up to 64 sequences).
+    // Warp-level form, one split a row: the CTA has the whole row in shared memory and writes the output itself (partial
+    // results and a merge kernel / so, us: 64 x 500 keys, 8 heads of 64 25.4 / 23.3; 40 x 3000, 64 / 32 heads of 64 97 / 94; 48 x
+    // 1500, 32 / 8 heads of 128 in 64-key tiles 43.8 / 41.0).  Not the tcgen05 form, whose rows end in tensor memory: read out
+    // by the few warps that may touch them, 64 x 2000 keys took 84 us in place of 60.
+    // The step merges a row's splits itself where its CTAs start together (one wave, or the shared-out form) and are more
+    // than two: a launch and the end of the grid less; us with a merge kernel and so: 1 sequence, 32 / 8 heads of 128, 4096
+    // keys 23.4 / 19.3, 64K keys 54 / 48; 3 sequences of 16K 39.8 / 37.0; heads of 64, 8192 keys 27.4 / 17.3; 16 ragged
+    // sequences shared out 76.5 / 74.6; two splits of 8 x 32K 124.3 / 125.2.  In a grid of several waves the merge at the end
+    // of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000, 32 KV heads 137 / 146.  Every such row needs
+    // a counter behind the status record (there are 248 with up to 64 sequences).
     const int words = static_cast<int>((kDecodeStatusBytes + decode_len_bytes(p->batch)) / 4) - 4, n_words = (prm.n_rows + 1) / 2;
     const bool umma = p->head_dim == 128 && p->tile_n == 128;
     const int64_t ctas = static_cast<int64_t>(g.n_splits) * prm.n_rows, wave = umma ? kDecodeWave : 2 * kDecodeWave;
-    prm.fused = n_words <= words && g.n_splits <= 0xffff && (g.balanced || (g.n_splits > 1 && ctas <= wave)) ? 1 : 0;
+    const bool counted = n_words <= words && g.n_splits <= 0xffff && (g.balanced || (g.n_splits > 2 && ctas <= wave));
+    prm.fused = counted || (!umma && g.n_splits == 1) ? 1 : 0;
     prm.arrived = reinterpret_cast<uint32_t*>(prm.status) + 4;
-    decode_prepare_kernel<<<1, 128, 0, s>>>(prm.status, prm.fused ? 4 + n_words : 4);
+    decode_prepare_kernel<<<1, 128, 0, s>>>(prm.status, counted ? 4 + n_words : 4);
     g_launch_count.fetch_add(1);
     cudaError_t pe = cudaGetLastError();
     if (pe != cudaSuccess) return static_cast<int>(pe);

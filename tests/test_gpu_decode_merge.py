@@ -1,4 +1,4 @@
-"""The merge of a decode step's splits inside the step (the CTAs of a row count their arrivals) on both sides of the line to the
+"""A row with one CTA, and the merge of splits inside the step (the CTAs of a row count their arrivals), on both sides of the line to the
 merge kernel: few and many splits, a last split of one tile, empty sequences, an odd number of rows (two rows share a counter
 word), repeated calls on one workspace whose counters hold garbage before each."""
 import numpy as np
@@ -13,6 +13,7 @@ DEV = "cuda:0"
 
 @pytest.mark.parametrize("B,Hq,Hk,d,tile,L,splits", [(1, 8, 1, 128, 128, 3000, 0), (3, 12, 3, 128, 128, 1100, 9), (3, 6, 3, 128, 128, 1500, -1),
                                                      (1, 4, 4, 64, 64, 4000, 0), (5, 10, 5, 64, 128, 700, 3), (3, 24, 3, 128, 64, 1000, 5),
+                                                     (5, 20, 5, 128, 128, 900, 1), (5, 40, 5, 128, 128, 700, 1), (5, 10, 5, 64, 128, 700, 1), (5, 10, 5, 128, 64, 400, 1), (5, 8, 2, 128, 128, 2000, -1),
                                                      (2, 148, 37, 128, 128, 300, 2), (2, 148, 74, 128, 128, 300, 2), (2, 75, 75, 64, 64, 500, 2)])
 def test_merge_in_the_step_against_the_oracle(B, Hq, Hk, d, tile, L, splits):
     from paper_2608_17336_b200 import binding as tm
