@@ -704,10 +704,10 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     const int R = p->heads_q / p->heads_kv;
     prm.out = static_cast<__half*>(out_f16);
     prm.lse = lse;
-    // Warp-level form, one split a row: the CTA has the whole row in shared memory and writes the output itself (partial
-    // results and a merge kernel / so, us: 64 x 500 keys, 8 heads of 64 25.4 / 23.3; 40 x 3000, 64 / 32 heads of 64 97 / 94; 48 x
-    // 1500, 32 / 8 heads of 128 in 64-key tiles 43.8 / 41.0).  Not the tcgen05 form, whose rows end in tensor memory: read out
-    // by the few warps that may touch them, 64 x 2000 keys took 84 us in place of 60.
+    // A row with one CTA needs no merge: that CTA writes the output, out of shared memory (warp-level form) or tensor memory
+    // (with partial results and a merge kernel / so, us: 64 x 500 keys, 8 heads of 64 25.4 / 23.3; 40 x 3000, 64 / 32 heads of
+    // 64 97 / 94; 48 x 1500, 32 / 8 heads of 128 in 64-key tiles 43.8 / 41.0; in 128-key tiles 64 x 2000 60.4 / 58.2, 16 x
+    // 16000 111.5 / 109.6).
     // The step merges a row's splits itself where its CTAs start together (one wave, or the shared-out form) and are more
     // than two: a launch and the end of the grid less; us with a merge kernel and so: 1 sequence, 32 / 8 heads of 128, 4096
     // keys 23.4 / 19.3, 64K keys 54 / 48; 3 sequences of 16K 39.8 / 37.0; heads of 64, 8192 keys 27.4 / 17.3; 16 ragged
@@ -718,7 +718,7 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     const bool umma = p->head_dim == 128 && p->tile_n == 128;
     const int64_t ctas = static_cast<int64_t>(g.n_splits) * prm.n_rows, wave = umma ? kDecodeWave : 2 * kDecodeWave;
     const bool counted = n_words <= words && g.n_splits <= 0xffff && (g.balanced || (g.n_splits > 2 && ctas <= wave));
-    prm.fused = counted || (!umma && g.n_splits == 1) ? 1 : 0;
+    prm.fused = counted || (!g.balanced && g.n_splits == 1) ? 1 : 0;
     prm.arrived = reinterpret_cast<uint32_t*>(prm.status) + 4;
     decode_prepare_kernel<<<1, 128, 0, s>>>(prm.status, counted ? 4 + n_words : 4);
     g_launch_count.fetch_add(1);

@@ -33,7 +33,7 @@ struct DecodeParams {
     __half* out;     // [B, Hq, D]
     float* lse;      // nullable [B, Hq]
     // 16 bits per (sequence, KV head) row, 0 before the step: CTAs of the row that have written their partial results.  The
-    // last one merges them.
+    // last one merges them.  (Not used by a row with one CTA, which writes the output itself.)
     uint32_t* arrived;
     int fused;       // 1: merged by the step, 0: by a kernel of its own
     int* status;     // 4 ints at the start of the workspace (same record as the attention kernel's)
@@ -78,22 +78,20 @@ __device__ __forceinline__ void merge_column(const DecodeParams& prm, int64_t ro
 }
 
 // At the end of a step's CTA, by all its threads, when the partial results that it owes have been stored: the last CTA of
-// row (b, hk) -- `ctas` of them -- merges the n_parts parts of its R query heads.
+// row (b, hk) -- `ctas` of them, two or more -- merges the n_parts parts of its R query heads.
 template <int D, int R>
 __device__ __forceinline__ void merge_if_last(const DecodeParams& prm, int b, int hk, int ctas, int n_parts) {
     __shared__ int last_s;
-    if (ctas > 1) __threadfence();        // this thread's partial results, before the arrival
+    __threadfence();        // this thread's partial results, before the arrival
     __syncthreads();
-    if (ctas > 1) {
-        if (threadIdx.x == 0) {
-            const int row = b * prm.Hk + hk;
-            const uint32_t before = atomicAdd(prm.arrived + (row >> 1), 1u << (16 * (row & 1)));
-            last_s = static_cast<int>((before >> (16 * (row & 1))) & 0xffffu) == ctas - 1;
-        }
-        __syncthreads();
-        if (!last_s) return;
-        __threadfence();
+    if (threadIdx.x == 0) {
+        const int row = b * prm.Hk + hk;
+        const uint32_t before = atomicAdd(prm.arrived + (row >> 1), 1u << (16 * (row & 1)));
+        last_s = static_cast<int>((before >> (16 * (row & 1))) & 0xffffu) == ctas - 1;
     }
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
     for (int i = threadIdx.x; i < R * D; i += blockDim.x)
         merge_column<D>(prm, static_cast<int64_t>(b) * prm.Hq + hk * R + i / D, n_parts, i % D);
 }

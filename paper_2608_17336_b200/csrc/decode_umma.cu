@@ -65,6 +65,7 @@ constexpr int kThreads = (kPvWarp + 1) * 32;
 constexpr int kConvThreads = kConvWarps * 32;
 constexpr int kTmemCols = 512;            // S^T: four buffers of 16 columns from column 0; O of stream g: 128 + 128 g
 constexpr uint32_t kColO = 128;
+constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kMoveAbove = 8.f;         // m moves when a step's maximum exceeds it by more than 2^8
 constexpr int kRowsPerLane = 5, kMaxRows = 32 * kRowsPerLane;   // rows of a batch whose splits one warp can balance
 
@@ -77,6 +78,7 @@ struct Small {
     uint32_t slot_info[kSlots];           // ring units of the tile in a slot: K (byte 0), second K slab (1), V (2)
     float warp_max[kStreams][kStreamWarps][8];
     float zsum[kStreams][kStreamWarps][8];
+    float m_end[kStreams][8], z_end[kStreams][8];   // one CTA per row: maximum and row sum of each stream
     float dq[8];
     uint32_t tmem_base;
     int abort_flag;
@@ -297,7 +299,13 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         }
     };
 
+    const bool alone = prm.fused && row_splits == 1;   // this CTA has the whole row: no partial results
     if (n_it <= 0) {                      // a split without keys: the merge skips it
+        if (alone) {
+            const int64_t head0 = static_cast<int64_t>(b) * prm.Hq + hk * R;
+            for (int idx = tid; idx < R * D; idx += kThreads) prm.out[head0 * D + idx] = __float2half_rn(0.f);
+            if (tid < R && prm.lse != nullptr) prm.lse[head0 + tid] = -INFINITY;
+        } else {
         for (int idx = tid; idx < kStreams * R * D; idx += kThreads) {
             const int g = idx / (R * D), rd = idx % (R * D);
             prm.o_part[(out_row0 + static_cast<int64_t>(rd / D) * n_parts + g) * D + (rd % D)] = 0.f;
@@ -306,9 +314,10 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
             prm.m_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = -INFINITY;
             prm.z_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = 0.f;
         }
+        }
         if (q_writer && warp < R) prep_query_row(warp, false);   // (a row without keys still reports its quantised query)
         leave();
-        if (prm.fused) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
+        if (prm.fused && !alone) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
         return;
     }
 
@@ -575,9 +584,12 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         const int64_t orow = out_row0 + static_cast<int64_t>(lane < R ? lane : 0) * n_parts + g;   // (lanes < R of quarter 0)
         if (g >= n_pairs) {
             // a stream without a step: an empty partial result, which the merge skips
-            for (int idx = key; idx < R * D; idx += kStreamWarps * 32)
+            for (int idx = key; !alone && idx < R * D; idx += kStreamWarps * 32)
                 prm.o_part[(out_row0 + static_cast<int64_t>(idx / D) * n_parts + g) * D + (idx % D)] = 0.f;
-            if (wq == 0 && lane < R) { prm.m_part[orow] = -INFINITY; prm.z_part[orow] = 0.f; }
+            if (wq == 0 && lane < R) {
+                if (alone) sh.m_end[g][lane] = -INFINITY;
+                else { prm.m_part[orow] = -INFINITY; prm.z_part[orow] = 0.f; }
+            }
         }
         for (int j = g; j < n_pairs; j += kStreams) {
             const uint32_t par = (j >> 1) & 1;        // phase parity of this stream's barriers at this step
@@ -698,7 +710,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 if (!wait(&sh.pv_pair[g], par, kWPV)) break;      // the PVs of this step
                 ptx::tc_fence_after_sync();
 #pragma unroll 1
-                for (int c = 0; c < D / 32; ++c) {
+                for (int c = 0; c < D / 32 && !alone; ++c) {
                     uint32_t o[32];
                     ptx::tmem_ld32(tmem_base + col_o + 32 * c, o);
                     ptx::tmem_wait_ld_dep(o);
@@ -714,8 +726,9 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                     float mine = -INFINITY;
 #pragma unroll
                     for (int r = 0; r < R; ++r) if (lane == r) mine = m_run[r];
-                    prm.m_part[orow] = mine;
-                    prm.z_part[orow] = sh.zsum[g][0][lane] + sh.zsum[g][1][lane] + sh.zsum[g][2][lane] + sh.zsum[g][3][lane];
+                    const float z_row = sh.zsum[g][0][lane] + sh.zsum[g][1][lane] + sh.zsum[g][2][lane] + sh.zsum[g][3][lane];
+                    if (alone) { sh.m_end[g][lane] = mine; sh.z_end[g][lane] = z_row; }
+                    else { prm.m_part[orow] = mine; prm.z_part[orow] = z_row; }
                 }
                 ptx::tc_fence_before_sync();
             }
@@ -736,12 +749,45 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 if (ptx::mbar_try_wait(ptx::smem_u32(&sh.full[it % kSlots]), (it / kSlots) & 1)) break;
         }
     }
+    if (alone && !*abort_flag && warp < 16 && (warp & 3) == 0) {
+        // The two streams' results out of tensor memory: rows are lanes 0..R-1 (which warps 4i may touch), a warp takes 32
+        // columns.  One factor a row and stream: with a division an element these four warps are a chain of latencies at the
+        // end of every CTA (64 sequences of up to 2000 keys 84 us; now 58.2, with a merge kernel 60.4).
+        ptx::tc_fence_after_sync();
+        const int r = lane < R ? lane : 0;
+        const float m0 = sh.m_end[0][r], m1 = sh.m_end[1][r], m = fmaxf(m0, m1);     // (stream 0 has a step)
+        const float w0 = exp2f(m0 - m), w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - m);
+        const float z = m1 == -INFINITY ? sh.z_end[0][r] * w0 : sh.z_end[0][r] * w0 + sh.z_end[1][r] * w1;
+        const float f0 = z > 0.f ? w0 / z : 0.f, f1 = z > 0.f ? w1 / z : 0.f;
+        const int64_t head = static_cast<int64_t>(b) * prm.Hq + hk * R + r;
+#pragma unroll 1
+        for (int c = 8 * warp; c < 8 * warp + 32; c += 8) {
+            uint32_t o0[8], o1[8];
+            ptx::tmem_ld32x32_x8(tmem_base + kColO + c, o0);
+            ptx::tmem_ld32x32_x8(tmem_base + kColO + 128 + c, o1);
+            ptx::tmem_wait_ld_dep(o0, o1);
+            __half2 h[4];
+#pragma unroll
+            for (int x = 0; x < 8; x += 2) {
+                float v[2];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    v[y] = __uint_as_float(o0[x + y]) * f0;
+                    if (f1 != 0.f) v[y] += __uint_as_float(o1[x + y]) * f1;
+                }
+                h[x / 2] = __floats2half2_rn(v[0], v[1]);
+            }
+            if (lane < R) *reinterpret_cast<uint4*>(prm.out + head * D + c) = *reinterpret_cast<const uint4*>(h);
+        }
+        if (warp == 0 && lane < R && prm.lse != nullptr) prm.lse[head] = z > 0.f ? (m + log2f(z)) * kLn2 : -INFINITY;
+        ptx::tc_fence_before_sync();
+    }
     __syncthreads();
     if (warp == kProducerWarp) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, kTmemCols);
     }
-    if (prm.fused && !*abort_flag) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
+    if (prm.fused && !alone && !*abort_flag) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
