@@ -97,7 +97,7 @@ __device__ __forceinline__ void merge_if_last(const DecodeParams& prm, int b, in
 }
 
 // The tcgen05 form of the step for head_dim 128, tile_n 128 (R = Hq / Hk in {1, 2, 4, 8}): enqueues the kernel
-// that writes (m, z, O~) of every split to the workspace; the caller launches the merge.  Returns a cudaError_t
+// that writes the output (prm.fused) or (m, z, O~) of every split to the workspace, for the caller's merge kernel.  Returns a cudaError_t
 // or a TILEMIX_ERR_* code.
 int launch_decode_umma(int R, const DecodeParams& prm, cudaStream_t stream);
 
