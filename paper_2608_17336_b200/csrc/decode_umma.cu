@@ -751,14 +751,17 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     }
     if (alone && !*abort_flag && warp < 16 && (warp & 3) == 0) {
         // The two streams' results out of tensor memory: rows are lanes 0..R-1 (which warps 4i may touch), a warp takes 32
-        // columns.  One factor a row and stream: with a division an element these four warps are a chain of latencies at the
-        // end of every CTA (64 sequences of up to 2000 keys 84 us; now 58.2, with a merge kernel 60.4).
+        // columns.  What the merge does with two parts: one whose maximum is -inf has no weight, whatever its row sum and its
+        // O hold, and a row whose sum is not positive is 0 with lse = -inf.
+        // One reciprocal a row: with a division an element these four warps are a chain of latencies at the end of every
+        // CTA (64 sequences of up to 2000 keys 84 us; now 58.2, with a merge kernel 60.4).
         ptx::tc_fence_after_sync();
         const int r = lane < R ? lane : 0;
-        const float m0 = sh.m_end[0][r], m1 = sh.m_end[1][r], m = fmaxf(m0, m1);     // (stream 0 has a step)
-        const float w0 = exp2f(m0 - m), w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - m);
-        const float z = m1 == -INFINITY ? sh.z_end[0][r] * w0 : sh.z_end[0][r] * w0 + sh.z_end[1][r] * w1;
-        const float f0 = z > 0.f ? w0 / z : 0.f, f1 = z > 0.f ? w1 / z : 0.f;
+        const float m0 = sh.m_end[0][r], m1 = sh.m_end[1][r], m = fmaxf(m0, m1);
+        float w0 = m0 == -INFINITY ? 0.f : exp2f(m0 - m), w1 = m1 == -INFINITY ? 0.f : exp2f(m1 - m);
+        const float z = (m0 == -INFINITY ? 0.f : sh.z_end[0][r] * w0) + (m1 == -INFINITY ? 0.f : sh.z_end[1][r] * w1);
+        if (!(z > 0.f)) w0 = w1 = 0.f;
+        const float rz = z > 0.f ? 1.f / z : 0.f;
         const int64_t head = static_cast<int64_t>(b) * prm.Hq + hk * R + r;
 #pragma unroll 1
         for (int c = 8 * warp; c < 8 * warp + 32; c += 8) {
@@ -772,8 +775,9 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 float v[2];
 #pragma unroll
                 for (int y = 0; y < 2; ++y) {
-                    v[y] = __uint_as_float(o0[x + y]) * f0;
-                    if (f1 != 0.f) v[y] += __uint_as_float(o1[x + y]) * f1;
+                    v[y] = w0 != 0.f ? __uint_as_float(o0[x + y]) * w0 : 0.f;
+                    if (w1 != 0.f) v[y] += __uint_as_float(o1[x + y]) * w1;
+                    v[y] *= rz;
                 }
                 h[x / 2] = __floats2half2_rn(v[0], v[1]);
             }
