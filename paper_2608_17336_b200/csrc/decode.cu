@@ -502,7 +502,7 @@ decode_kernel(const DecodeParams prm) {
             if (e == 0) { prm.m_part[part] = m; prm.z_part[part] = z; }
         }
     }
-    if (prm.fused && prm.n_splits > 1) merge_if_last<D, R>(prm, b, hk, prm.n_splits, prm.n_splits);
+    if (prm.fused && prm.n_splits > 1) merge_if_last<D, R, kDecodeThreads>(prm, b, hk, prm.n_splits, prm.n_splits);
 }
 
 // Merge as a kernel of its own (grids of several waves, see tilemix_decode_int8kv): one block per query head, one thread per
@@ -511,7 +511,7 @@ template <int D>
 __global__ void __launch_bounds__(D)
 decode_merge_kernel(const DecodeParams prm) {
     ptx::griddep_wait();   // (when launched as a programmatic dependent of the step kernel)
-    merge_column<D>(prm, blockIdx.x, prm.n_parts, threadIdx.x);
+    merge_columns<D, 1>(prm, blockIdx.x, prm.n_parts, threadIdx.x);
 }
 
 // Step and merge overlap the tail of the kernel before them (programmatic dependent launch).
@@ -575,6 +575,7 @@ size_t decode_len_bytes(int B) { return (static_cast<size_t>(B) * sizeof(int32_t
 
 struct DecodeGeometry {
     int n_blk, T_mask, W, n_splits;
+    int k_tiles;            // kernel tiles of a row of max_len keys
     int n_parts;            // partial results per query head in the workspace (the tcgen05 form writes two per split)
     int balanced, n_ctas, split_cap;   // tcgen05 form with an automatic split count: see DecodeParams
     size_t o_bytes, mz_bytes;
@@ -645,6 +646,7 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
     if (splits > 65535) return TILEMIX_ERR_UNSUPPORTED;
     if (splits > k_tiles) splits = k_tiles;      // a split is whole kernel tiles: more of them would only be empty CTAs
     g->n_splits = splits;
+    g->k_tiles = k_tiles;
     g->n_parts = umma ? 2 * (g->balanced ? g->split_cap : splits) : splits;
     const size_t rows = static_cast<size_t>(p->batch) * p->heads_q * g->n_parts;
     g->o_bytes = (rows * p->head_dim * sizeof(float) + 255) / 256 * 256;
@@ -708,19 +710,24 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     // (with partial results and a merge kernel / so, us: 64 x 500 keys, 8 heads of 64 25.4 / 23.3; 40 x 3000, 64 / 32 heads of
     // 64 97 / 94; 48 x 1500, 32 / 8 heads of 128 in 64-key tiles 43.8 / 41.0; in 128-key tiles 64 x 2000 60.4 / 58.2, 16 x
     // 16000 111.5 / 109.6).
-    // The step merges a row's splits itself where its CTAs start together (one wave, or the shared-out form) and are more
-    // than two: a launch and the end of the grid less; us with a merge kernel and so: 1 sequence, 32 / 8 heads of 128, 4096
-    // keys 23.4 / 19.3, 64K keys 54 / 48; 3 sequences of 16K 39.8 / 37.0; heads of 64, 8192 keys 27.4 / 17.3; 16 ragged
-    // sequences shared out 76.5 / 74.6; two splits of 8 x 32K 124.3 / 125.2.  In a grid of several waves the merge at the end
-    // of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000, 32 KV heads 137 / 146.  Every such row needs
-    // a counter behind the status record (there are 248 with up to 64 sequences).
+    // Of a row with more CTAs the last one merges at its end, where they start together (one wave, or the shared-out form) and
+    // are more than two: no third kernel behind the end of the grid.  us with the merge kernel and so (calls in one CUDA
+    // graph), 128-key tiles of 128: one sequence, 8 KV heads, four query heads each, 8000 keys 19.6 / 19.1, 40000 keys 35.5 /
+    // 34.7, eight each 42.2 / 40.6; 12 x 2500 keys, 4 KV heads 20.5 / 20.0; heads of 64: one sequence, 3072 keys 9.7 / 9.1,
+    // 42 rows x 5000 keys, eight query heads 18.6 / 17.6.  Two splits: 64 rows x 2048 keys, 128-key tiles of 128 19.5 / 18.6,
+    // x 4096 28.3 / 28.2, 128 rows x 2048 keys of 64 17.75 / 18.1, x 8192 48.3 / 48.3: those keep the kernel.  So do three
+    // and four splits of two kernel tiles in the warp-level form: so short a step ends before the merge has got under way
+    // (one sequence, 384 keys of 128 in 64-key tiles 8.7 / 9.6, 768 keys of 64 8.2 / 9.0).  In a grid of several waves the merge
+    // at the end of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000, 32 KV heads 137 / 146.  Every
+    // row merged so needs a counter behind the status record (there are 248 with up to 64 sequences).
     const int words = static_cast<int>((kDecodeStatusBytes + decode_len_bytes(p->batch)) / 4) - 4, n_words = (prm.n_rows + 1) / 2;
     const bool umma = p->head_dim == 128 && p->tile_n == 128;
     const int64_t ctas = static_cast<int64_t>(g.n_splits) * prm.n_rows, wave = umma ? kDecodeWave : 2 * kDecodeWave;
-    const bool counted = n_words <= words && g.n_splits <= 0xffff && (g.balanced || (g.n_splits > 2 && ctas <= wave));
+    const bool in_step = g.n_splits > 2 && ctas <= wave && (umma || g.n_splits > 4 || g.k_tiles > 2 * g.n_splits);
+    const bool counted = n_words <= words && g.n_splits <= 0xffff && (g.balanced || in_step);
     prm.fused = counted || (!g.balanced && g.n_splits == 1) ? 1 : 0;
     prm.arrived = reinterpret_cast<uint32_t*>(prm.status) + 4;
-    decode_prepare_kernel<<<1, 128, 0, s>>>(prm.status, counted ? 4 + n_words : 4);
+    decode_prepare_kernel<<<1, counted ? 128 : 32, 0, s>>>(prm.status, counted ? 4 + n_words : 4);
     g_launch_count.fetch_add(1);
     cudaError_t pe = cudaGetLastError();
     if (pe != cudaSuccess) return static_cast<int>(pe);

@@ -42,15 +42,18 @@ struct DecodeParams {
 };
 
 // Merge of partial results: m = max m_s, z = sum z_s 2^(m_s - m), O = sum O~_s 2^(m_s - m) / z for the query head `row` of
-// [B, Hq] and output column e; a whole warp with consecutive columns.  The parts are taken 32 at a time: lane s loads
-// (m_s, z_s) and the weights are shared by shuffles, so that the loads of O~_s depend on one round trip only and are in
-// flight together (a part that nobody wrote has m_s = -inf, weight 0, and is not loaded).
-template <int D>
-__device__ __forceinline__ void merge_column(const DecodeParams& prm, int64_t row, int n_parts, int e) {
+// [B, Hq] and the C output columns from e on; a whole warp with consecutive columns.  The parts are taken 32 at a time: lane
+// s loads (m_s, z_s) and the weights are shared by shuffles, so that the loads of O~_s depend on one round trip only and are
+// in flight together (a part that nobody wrote has m_s = -inf, weight 0, and is not loaded).
+template <int D, int C>
+__device__ __forceinline__ void merge_columns(const DecodeParams& prm, int64_t row, int n_parts, int e) {
+    static_assert(C == 1 || C == 2 || C == 4, "one load per part");
     constexpr float kLn2f = 0.6931471805599453f;
     const int lane = threadIdx.x & 31;
     const int64_t first = row * prm.n_parts;
-    float m = -INFINITY, z = 0.f, o = 0.f;
+    float m = -INFINITY, z = 0.f, o[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) o[c] = 0.f;
     for (int s0 = 0; s0 < n_parts; s0 += 32) {
         const int s = s0 + lane;
         const float ms = s < n_parts ? __ldcg(prm.m_part + first + s) : -INFINITY;
@@ -63,24 +66,47 @@ __device__ __forceinline__ void merge_column(const DecodeParams& prm, int64_t ro
         const float back = m == -INFINITY ? 0.f : exp2f(m - m_new);
         const float w = ms == -INFINITY ? 0.f : exp2f(ms - m_new);
         const float zw = ms == -INFINITY ? 0.f : zs * w;
-        z *= back; o *= back; m = m_new;
-        const int cnt = min(32, n_parts - s0);
+        z *= back; m = m_new;
+#pragma unroll
+        for (int c = 0; c < C; ++c) o[c] *= back;
         const float* src = prm.o_part + (first + s0) * D + e;
-#pragma unroll 8
-        for (int i = 0; i < cnt; ++i) {
-            const float wi = __shfl_sync(0xffffffffu, w, i);
-            z += __shfl_sync(0xffffffffu, zw, i);
-            if (wi != 0.f) o += __ldcg(src + static_cast<int64_t>(i) * D) * wi;
+        // eight at a time, the last group too: the lanes past the last part hold weight 0 (one part after the other at the
+        // end is a chain of round trips, and a row of a few splits has nothing else)
+        for (int i0 = 0; i0 < min(32, n_parts - s0); i0 += 8) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float wi = __shfl_sync(0xffffffffu, w, i0 + k);
+                z += __shfl_sync(0xffffffffu, zw, i0 + k);
+                if (wi != 0.f) {
+                    alignas(16) float x[C];
+                    const float* at = src + static_cast<int64_t>(i0 + k) * D;
+                    if constexpr (C == 4) *reinterpret_cast<float4*>(x) = __ldcg(reinterpret_cast<const float4*>(at));
+                    else if constexpr (C == 2) *reinterpret_cast<float2*>(x) = __ldcg(reinterpret_cast<const float2*>(at));
+                    else x[0] = __ldcg(at);
+#pragma unroll
+                    for (int c = 0; c < C; ++c) o[c] += x[c] * wi;
+                }
+            }
         }
     }
-    prm.out[row * D + e] = __float2half_rn(z > 0.f ? o / z : 0.f);
+    alignas(8) __half h[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) h[c] = __float2half_rn(z > 0.f ? o[c] / z : 0.f);
+    __half* dst = prm.out + row * D + e;
+    if constexpr (C == 4) *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(h);
+    else if constexpr (C == 2) *reinterpret_cast<__half2*>(dst) = *reinterpret_cast<const __half2*>(h);
+    else dst[0] = h[0];
     if (e == 0 && prm.lse != nullptr) prm.lse[row] = z > 0.f ? (m + log2f(z)) * kLn2f : -INFINITY;
 }
 
-// At the end of a step's CTA, by all its threads, when the partial results that it owes have been stored: the last CTA of
-// row (b, hk) -- `ctas` of them, two or more -- merges the n_parts parts of its R query heads.
-template <int D, int R>
+// At the end of a step's CTA of THREADS threads, by all of them, when the partial results that it owes have been stored: the
+// last CTA of row (b, hk) -- `ctas` of them, two or more -- merges the n_parts parts of its R query heads.  A thread takes as
+// many adjacent columns as let one pass do: another pass is two more round trips to L2 behind the first (8 query heads of 128 in
+// 64-key tiles, one sequence of 8000 keys: four passes 29.4 us, one 15.5, merge kernel 22.9).
+template <int D, int R, int THREADS>
 __device__ __forceinline__ void merge_if_last(const DecodeParams& prm, int b, int hk, int ctas, int n_parts) {
+    constexpr int C = R * D <= THREADS ? 1 : R * D <= 2 * THREADS ? 2 : 4;
+    static_assert(R * D <= C * THREADS && D % (32 * C) == 0, "one pass, a warp inside one row");
     __shared__ int last_s;
     __threadfence();        // this thread's partial results, before the arrival
     __syncthreads();
@@ -92,8 +118,8 @@ __device__ __forceinline__ void merge_if_last(const DecodeParams& prm, int b, in
     __syncthreads();
     if (!last_s) return;
     __threadfence();
-    for (int i = threadIdx.x; i < R * D; i += blockDim.x)
-        merge_column<D>(prm, static_cast<int64_t>(b) * prm.Hq + hk * R + i / D, n_parts, i % D);
+    const int i = C * threadIdx.x;
+    if (i < R * D) merge_columns<D, C>(prm, static_cast<int64_t>(b) * prm.Hq + hk * R + i / D, n_parts, i % D);
 }
 
 // The tcgen05 form of the step for head_dim 128, tile_n 128 (R = Hq / Hk in {1, 2, 4, 8}): enqueues the kernel

@@ -317,7 +317,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         }
         if (q_writer && warp < R) prep_query_row(warp, false);   // (a row without keys still reports its quantised query)
         leave();
-        if (prm.fused && !alone) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
+        if (prm.fused && !alone) merge_if_last<D, R, kThreads>(prm, b, hk, row_splits, kStreams * row_splits);
         return;
     }
 
@@ -791,7 +791,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, kTmemCols);
     }
-    if (prm.fused && !alone && !*abort_flag) merge_if_last<D, R>(prm, b, hk, row_splits, kStreams * row_splits);
+    if (prm.fused && !alone && !*abort_flag) merge_if_last<D, R, kThreads>(prm, b, hk, row_splits, kStreams * row_splits);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
