@@ -710,21 +710,23 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     // (with partial results and a merge kernel / so, us: 64 x 500 keys, 8 heads of 64 25.4 / 23.3; 40 x 3000, 64 / 32 heads of
     // 64 97 / 94; 48 x 1500, 32 / 8 heads of 128 in 64-key tiles 43.8 / 41.0; in 128-key tiles 64 x 2000 60.4 / 58.2, 16 x
     // 16000 111.5 / 109.6).
-    // Of a row with more CTAs the last one merges at its end, where they start together (one wave, or the shared-out form) and
-    // are more than two: no third kernel behind the end of the grid.  us with the merge kernel and so (calls in one CUDA
-    // graph), 128-key tiles of 128: one sequence, 8 KV heads, four query heads each, 8000 keys 19.6 / 19.1, 40000 keys 35.5 /
-    // 34.7, eight each 42.2 / 40.6; 12 x 2500 keys, 4 KV heads 20.5 / 20.0; heads of 64: one sequence, 3072 keys 9.7 / 9.1,
-    // 42 rows x 5000 keys, eight query heads 18.6 / 17.6.  Two splits: 64 rows x 2048 keys, 128-key tiles of 128 19.5 / 18.6,
-    // x 4096 28.3 / 28.2, 128 rows x 2048 keys of 64 17.75 / 18.1, x 8192 48.3 / 48.3: those keep the kernel.  So do three
-    // and four splits of two kernel tiles in the warp-level form: so short a step ends before the merge has got under way
-    // (one sequence, 384 keys of 128 in 64-key tiles 8.7 / 9.6, 768 keys of 64 8.2 / 9.0).  In a grid of several waves the merge
-    // at the end of a CTA holds up the one behind it: 64 x 2000 keys 60.4 / 62.7, 32 x 4000, 32 KV heads 137 / 146.  Every
-    // row merged so needs a counter behind the status record (there are 248 with up to 64 sequences).
-    const int words = static_cast<int>((kDecodeStatusBytes + decode_len_bytes(p->batch)) / 4) - 4, n_words = (prm.n_rows + 1) / 2;
+    // Of a row with more CTAs the last one merges at its end, where they start together (one wave; the shared-out form, in
+    // its two waves too: 16 ragged sequences 76.5 / 74.6) and are more than two: no third kernel behind the end of the grid.
+    // us with the merge kernel and so (calls in one CUDA graph), 128-key tiles of 128: one sequence, 8 KV heads, four query
+    // heads each, 8000 keys 19.6 / 19.1, 40000 keys 35.5 / 34.7, eight each 42.2 / 40.6; 12 x 2500 keys, 4 KV heads 20.5 /
+    // 20.0; heads of 64: one sequence, 3072 keys 9.7 / 9.1, 42 rows x 5000 keys, eight query heads 18.6 / 17.6.  Two splits:
+    // 64 rows x 2048 keys, 128-key tiles of 128 19.5 / 18.6, x 4096 28.3 / 28.2, 128 rows x 2048 keys of 64 17.75 / 18.1, x
+    // 8192 48.3 / 48.3: those keep the kernel.  So do three and four splits of two kernel tiles in the warp-level form: so
+    // short a step ends before the merge has got under way (one sequence, 384 keys of 128 in 64-key tiles 8.7 / 9.6, 768
+    // keys of 64 8.2 / 9.0).  In a grid of several waves the merge at the end of a CTA holds up the one behind it: 64 x 2000
+    // keys 60.4 / 62.7, 32 x 4000, 32 KV heads 137 / 146.  Every row merged so has a counter behind the status record.
     const bool umma = p->head_dim == 128 && p->tile_n == 128;
     const int64_t ctas = static_cast<int64_t>(g.n_splits) * prm.n_rows, wave = umma ? kDecodeWave : 2 * kDecodeWave;
     const bool in_step = g.n_splits > 2 && ctas <= wave && (umma || g.n_splits > 4 || g.k_tiles > 2 * g.n_splits);
-    const bool counted = n_words <= words && g.n_splits <= 0xffff && (g.balanced || in_step);
+    const bool counted = g.balanced || in_step;
+    // 16 bits a row, of at most one wave's rows: the shared-out form has no more, more than two splits in two waves are 98
+    static_assert(4 + (kDecodeWave + 1) / 2 <= static_cast<int>(kDecodeStatusBytes + 256) / 4, "the counters lie behind the status record");
+    const int n_words = (prm.n_rows + 1) / 2;
     prm.fused = counted || (!g.balanced && g.n_splits == 1) ? 1 : 0;
     prm.arrived = reinterpret_cast<uint32_t*>(prm.status) + 4;
     decode_prepare_kernel<<<1, counted ? 128 : 32, 0, s>>>(prm.status, counted ? 4 + n_words : 4);

@@ -261,13 +261,6 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     // shared memory (to_smem), and -- from the one split of the row that starts at its first group -- the quantised
     // row and its scale to the caller's buffers.
     const bool q_writer = g0 == 0 && (g1 > 0 || split + 1 == row_splits);
-    // (merged by a kernel of its own) parts of the row that no split writes (balanced form: the row has fewer splits than the workspace has room
-    // for): marked empty for the merge by the row's first split
-    if (split == 0 && !prm.fused)
-        for (int idx = tid; idx < R * (n_parts - kStreams * row_splits); idx += kThreads) {
-            const int r = idx / (n_parts - kStreams * row_splits), part = kStreams * row_splits + idx % (n_parts - kStreams * row_splits);
-            prm.m_part[(static_cast<int64_t>(b) * prm.Hq + hk * R + r) * n_parts + part] = -INFINITY;
-        }
     auto prep_query_row = [&](int r, bool to_smem) {
         const int hq = hk * R + r;
         const __half* qrow = prm.q + (static_cast<int64_t>(b) * prm.Hq + hq) * D;
