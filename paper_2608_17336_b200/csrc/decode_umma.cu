@@ -84,13 +84,21 @@ struct Small {
     int abort_flag;
     int row_cost[kMaxRows];               // balanced splits: cost of every (sequence, KV head) row of the batch
     int asg[4];                           // ... and this CTA's row, split and the row's number of splits
+    int item[4];                          // sequence, KV head, splits of the row
 };
 constexpr int kSmemBytes = kOffSmall + static_cast<int>(sizeof(Small)) + 1024;   // + slack to align the base to 1 KB
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 
 enum Which : int { kWFull = 1, kWFree = 2, kWS = 3, kWSFree = 4, kWP = 5, kWV = 6, kWPV = 7, kWXchg = 8, kWDrain = 9 };
 
-template <int R, bool F16K>
+// How a CTA's results leave: as partial results for the merge kernel; as output, by the one CTA of a row; or either, the
+// row's last CTA merging the partial results (the shared-out form: rows of one CTA and of several).  Instances of their own:
+// with all three in one kernel what only one of them needs at the end was carried through the softmax loop and spilled there
+// (8 KV heads of eight query heads each, 8 x 32K keys 141 us, 138 so, 16 x 16000 132 and 117; of four each 16 x 16000 103.0
+// and 102.5; of two each 64 sequences of up to 2000 keys 52.6 and 50.6).
+enum End : int { kEndPartial, kEndAlone, kEndInStep };
+
+template <int R, bool F16K, int END>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_constant__ CUtensorMap tm_k16,
                    const DecodeParams prm) {
@@ -292,25 +300,27 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         }
     };
 
-    const bool alone = prm.fused && row_splits == 1;   // this CTA has the whole row: no partial results
-    if (n_it <= 0) {                      // a split without keys: the merge skips it
+    const bool alone = END == kEndAlone || (END == kEndInStep && row_splits == 1);   // this CTA has the whole row: no partial results
+    volatile int* item_s = sh.item;       // read back where the CTA ends
+    if (END == kEndInStep && tid == 0) { item_s[0] = b; item_s[1] = hk; item_s[2] = row_splits; }
+    if (n_it <= 0) {                      // no keys: zeros, or a part that the merge skips
         if (alone) {
             const int64_t head0 = static_cast<int64_t>(b) * prm.Hq + hk * R;
             for (int idx = tid; idx < R * D; idx += kThreads) prm.out[head0 * D + idx] = __float2half_rn(0.f);
             if (tid < R && prm.lse != nullptr) prm.lse[head0 + tid] = -INFINITY;
         } else {
-        for (int idx = tid; idx < kStreams * R * D; idx += kThreads) {
-            const int g = idx / (R * D), rd = idx % (R * D);
-            prm.o_part[(out_row0 + static_cast<int64_t>(rd / D) * n_parts + g) * D + (rd % D)] = 0.f;
-        }
-        if (tid < kStreams * R) {
-            prm.m_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = -INFINITY;
-            prm.z_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = 0.f;
-        }
+            for (int idx = tid; idx < kStreams * R * D; idx += kThreads) {
+                const int g = idx / (R * D), rd = idx % (R * D);
+                prm.o_part[(out_row0 + static_cast<int64_t>(rd / D) * n_parts + g) * D + (rd % D)] = 0.f;
+            }
+            if (tid < kStreams * R) {
+                prm.m_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = -INFINITY;
+                prm.z_part[out_row0 + static_cast<int64_t>(tid % R) * n_parts + tid / R] = 0.f;
+            }
         }
         if (q_writer && warp < R) prep_query_row(warp, false);   // (a row without keys still reports its quantised query)
         leave();
-        if (prm.fused && !alone) merge_if_last<D, R, kThreads>(prm, b, hk, row_splits, kStreams * row_splits);
+        if (END == kEndInStep && !alone) merge_if_last<D, R, kThreads>(prm, b, hk, row_splits, kStreams * row_splits);
         return;
     }
 
@@ -336,7 +346,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         }
     }
 
-    ptx::griddep_launch_dependents();     // the merge kernel may be brought in; it waits for this grid to finish
+    ptx::griddep_launch_dependents();     // a merge kernel may be brought in; it waits for this grid to finish
     volatile int* abort_flag = &sh.abort_flag;
 
     // Bounded wait on one mbarrier phase; false when the CTA is giving up.
@@ -688,7 +698,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
             ptx::fence_proxy_async_smem();
             ptx::mbar_arrive(ptx::smem_u32(&sh.p_ready[g]));
             if (j + kStreams >= n_pairs) {
-                // ---- the stream's last step: (m, z, O~) to the workspace
+                // ---- the stream's last step: (m, z, O~) to the workspace, or (m, z) to the end of the CTA
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     float z = z_part[r];
@@ -702,7 +712,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 if (!wait(&sh.zbar[g], 0, kWXchg)) break;
                 if (!wait(&sh.pv_pair[g], par, kWPV)) break;      // the PVs of this step
                 ptx::tc_fence_after_sync();
-#pragma unroll 1
+    #pragma unroll 1
                 for (int c = 0; c < D / 32 && !alone; ++c) {
                     uint32_t o[32];
                     ptx::tmem_ld32(tmem_base + col_o + 32 * c, o);
@@ -730,8 +740,8 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
     }
 
     // ---- every role is out of its loop ---------------------------------------------------------------------
-    // The prepare kernel has completed before this grid does: the merge kernel waits for this grid only, and what the
-    // stream runs behind it may read the status record or use the workspace again.
+    // The prepare kernel has completed before this grid does, and before the row's counter is used: a merge kernel waits for
+    // this grid only, and what the stream runs behind it may read the status record or use the workspace again.
     ptx::griddep_wait();
     __syncthreads();
     if (*abort_flag && warp == kProducerWarp && lane == 0) {
@@ -742,7 +752,10 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 if (ptx::mbar_try_wait(ptx::smem_u32(&sh.full[it % kSlots]), (it / kSlots) & 1)) break;
         }
     }
-    if (alone && !*abort_flag && warp < 16 && (warp & 3) == 0) {
+    const int b_end = END == kEndInStep ? item_s[0] : b, hk_end = END == kEndInStep ? item_s[1] : hk;
+    const int splits_end = END == kEndInStep ? item_s[2] : row_splits;
+    const bool alone_end = END == kEndAlone || (END == kEndInStep && splits_end == 1);
+    if (alone_end && !*abort_flag && warp < 16 && (warp & 3) == 0) {
         // The two streams' results out of tensor memory: rows are lanes 0..R-1 (which warps 4i may touch), a warp takes 32
         // columns.  What the merge does with two parts: one whose maximum is -inf has no weight, whatever its row sum and its
         // O hold, and a row whose sum is not positive is 0 with lse = -inf.
@@ -755,7 +768,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         const float z = (m0 == -INFINITY ? 0.f : sh.z_end[0][r] * w0) + (m1 == -INFINITY ? 0.f : sh.z_end[1][r] * w1);
         if (!(z > 0.f)) w0 = w1 = 0.f;
         const float rz = z > 0.f ? 1.f / z : 0.f;
-        const int64_t head = static_cast<int64_t>(b) * prm.Hq + hk * R + r;
+        const int64_t head = static_cast<int64_t>(b_end) * prm.Hq + hk_end * R + r;
 #pragma unroll 1
         for (int c = 8 * warp; c < 8 * warp + 32; c += 8) {
             uint32_t o0[8], o1[8];
@@ -784,7 +797,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc(tmem_base, kTmemCols);
     }
-    if (prm.fused && !alone && !*abort_flag) merge_if_last<D, R, kThreads>(prm, b, hk, row_splits, kStreams * row_splits);
+    if (END == kEndInStep && !alone_end && !*abort_flag) merge_if_last<D, R, kThreads>(prm, b_end, hk_end, splits_end, kStreams * splits_end);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -806,9 +819,9 @@ int encode_cache_map(EncodeTiledFn enc, CUtensorMap* tm, const void* base, int e
                                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE));
 }
 
-template <int R>
-int launch_r(const DecodeParams& prm, const CUtensorMap& tk8, const CUtensorMap& tk16, cudaStream_t stream) {
-    auto kernel = prm.k16 != nullptr ? decode_umma_kernel<R, true> : decode_umma_kernel<R, false>;
+template <int R, int END>
+int launch_end(const DecodeParams& prm, const CUtensorMap& tk8, const CUtensorMap& tk16, cudaStream_t stream) {
+    auto kernel = prm.k16 != nullptr ? decode_umma_kernel<R, true, END> : decode_umma_kernel<R, false, END>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);   // (of the current context)
     if (e != cudaSuccess) return static_cast<int>(e);
     const dim3 grid = prm.balanced ? dim3(prm.n_ctas) : dim3(prm.n_splits, prm.Hk, prm.B);
@@ -822,6 +835,13 @@ int launch_r(const DecodeParams& prm, const CUtensorMap& tk8, const CUtensorMap&
     e = cudaLaunchKernelEx(&cfg, kernel, tk8, tk16, prm);
     g_launch_count.fetch_add(1);
     return static_cast<int>(e);
+}
+
+template <int R>
+int launch_r(const DecodeParams& prm, const CUtensorMap& tk8, const CUtensorMap& tk16, cudaStream_t stream) {
+    if (!prm.fused) return launch_end<R, kEndPartial>(prm, tk8, tk16, stream);
+    if (!prm.balanced && prm.n_splits == 1) return launch_end<R, kEndAlone>(prm, tk8, tk16, stream);
+    return launch_end<R, kEndInStep>(prm, tk8, tk16, stream);
 }
 
 }  // namespace
