@@ -72,8 +72,10 @@ constexpr float kLn2 = 0.6931471805599453f;
 // A redone step costs its tile a second pass and a wait for the PV in flight, and with 128 rows that move m on their own
 // account it is hardly ever one row's affair: kAccept is half of what FP16 holds, not less (at 2^8, 32 heads x 8K with
 // outlier channels took 628 us in place of 590; maps and inputs whose m rarely moves take the same time).
-// An INT8 value cache multiplies P by its block's scale before it is rounded, up to 65504 / 127: kAcceptScaled.
-constexpr float kAccept = 32768.f, kAcceptScaled = 256.f, kMove = 4.0f, kMargin = 6.0f;
+// An INT8 value cache multiplies P by its block's scale before it is rounded, up to 65504 / 127 = 516 where the values were
+// FP16: kAcceptScaled keeps that product below 33 020.
+constexpr float kAccept = 32768.f, kAcceptScaled = 64.f, kMove = 4.0f, kMargin = 6.0f;
+static_assert(kAcceptScaled * (65504.f / 127.f) < 65504.f, "scaled probabilities of an accepted step are finite in FP16");
 
 enum Role : int { kRoleSoftmaxA = 0, kRoleSoftmaxB = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQuant = 4 };
 enum Bar : int { kBarQ = 0, kBarRingFull = 1, kBarRingEmpty = 2, kBarS = 3, kBarP = 4, kBarO = 5, kBarDrain = 6, kBarPV = 7,
