@@ -11,7 +11,7 @@
 //                                       kind::i8 or kind::f16 by the tile's routing bit.
 //   P[R x 128 keys]                     2^(s - m) * delta_V rounded to FP16, written by the key's thread into a
 //                                       K-major operand tile; the row maximum m is shared by a stream's four warps
-//                                       and lazy: it moves only when a step's maximum exceeds it by 2^8.
+//                                       and lazy: it moves only when a step's maximum exceeds it by 2^6.
 //   V16[64 keys x 128] = FP16(V8)       two groups of eight warps convert the INT8 rows exactly (1024 + (x + 128) as
 //                                       FP16 bits, minus 1152), half a tile each, into the MN-major swizzled layout.
 //   O[64 x 128] (+)= P V16              kind::f16, accumulator in tensor memory; rows 0..R-1 are the output.
@@ -66,7 +66,9 @@ constexpr int kConvThreads = kConvWarps * 32;
 constexpr int kTmemCols = 512;            // S^T: four buffers of 16 columns from column 0; O of stream g: 128 + 128 g
 constexpr uint32_t kColO = 128;
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kMoveAbove = 8.f;         // m moves when a step's maximum exceeds it by more than 2^8
+constexpr float kMoveAbove = 6.f;         // m moves when a step's maximum exceeds it by more than 2^6
+// (a probability times its block's scale, at most 65504 / 127 where the values were FP16, is rounded to FP16)
+static_assert(64.f * (65504.f / 127.f) < 65504.f && kMoveAbove <= 6.f, "scaled probabilities are finite in FP16");
 constexpr int kRowsPerLane = 5, kMaxRows = 32 * kRowsPerLane;   // rows of a batch whose splits one warp can balance
 
 struct Small {
