@@ -918,7 +918,8 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                 if (mine) {
                     // (One copy of the half's code, or two: the issuers of the on-the-fly and packed-batch instances, which share
                     // their schedulers and the instruction cache with more code, are faster with one -- 32 / 8 heads, 8K on the
-                    // fly 616 -> 596 us, packed batch of 16 prompts 477 -> 468 -- the others with two: 32K 6470, with one 6570.)
+                    // fly 616 -> 596 us, packed batch of 16 prompts 477 -> 468 -- the others with two: 32K 6470, with one 6570.  Packed with
+                    // 64-dimensional heads takes the same time with either: 32 / 8 heads 446 -> 444, 64 / 8 807 -> 810, 32 / 32 523.)
 #pragma unroll (OTF || VL ? 1 : 2)
                     for (int h = 0; h < 2; ++h) {
                         if (SUB && 2 * j + h >= u_t) break;

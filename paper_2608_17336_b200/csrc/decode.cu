@@ -238,7 +238,7 @@ decode_kernel(const DecodeParams prm) {
     } else {
         __syncthreads();   // barriers initialised, query rows and tile metadata staged
     }
-    ptx::griddep_launch_dependents();     // the merge kernel may be brought in; it waits for this grid to finish
+    ptx::griddep_launch_dependents();     // a merge kernel may be brought in; it waits for this grid to finish
 
     // per-warp flash-decoding state: rows g (< R) of this warp's keys
     float m_run = -INFINITY, z_part = 0.f;          // z_part: this lane's share of the row sum
@@ -435,10 +435,10 @@ decode_kernel(const DecodeParams prm) {
         }
     }
 
-    // ---- merge of the eight warps, then (m, z, O~) of this split to the workspace --------------------
+    // ---- merge of the eight warps; the row's only split writes the output, others (m, z, O~) to the workspace -----
     __syncthreads();   // every warp is out of the ring (all copies it waited for have landed)
-    // The prepare kernel has completed before this grid does: the merge kernel waits for this grid only, and what the
-    // stream runs behind it may read the status record or use the workspace again.
+    // The prepare kernel has completed before this grid does, and before the row's counter is used: a merge kernel waits for
+    // this grid only, and what the stream runs behind it may read the status record or use the workspace again.
     ptx::griddep_wait();
     if (*reinterpret_cast<volatile int*>(&abort_flag)) {
         if (tid == 0 && atomicCAS(&prm.status[0], 0, TILEMIX_ERR_DEVICE_TIMEOUT) == 0) {
@@ -614,8 +614,10 @@ int resolve_decode(const tilemix_decode_t* p, DecodeGeometry* g) {
             if (splits > cap) splits = cap;
             // On request, for a batch whose rows fit one wave: the kernel shares the wave's CTAs out by the rows'
             // cost (cache length, FP16-routed groups), up to split_cap to a row; the workspace has room for that
-            // many.  Not the default: with rows of one length it gains ~3 % (the FP16-routed groups differ) and
-            // loses ~5 us -- a full wave leaves no SM on which the merge kernel can wait ahead of time.
+            // many.  Not the default: rows of one length get the same number of CTAs that way, or two waves of them, and
+            // pay for the sharing out (us uniform / shared out: 8 x 8 rows of 32K keys 110 / 118, of 8K 39 / 45, 4 x 8 of 32K
+            // 63 / 71, 16 x 8 of 12K 80 / 107, one sequence of 64K 43 / 49); and which keys a CTA gets then depends on the
+            // lengths beside it.
             if (balance && n_rows <= kDecodeWave && n_rows <= kDecodeBalanceRows) {
                 int row_cap = 8 * splits < 16 ? 16 : 8 * splits;
                 if (row_cap > cap) row_cap = cap;
@@ -734,7 +736,7 @@ int tilemix_decode_int8kv(const tilemix_decode_t* p, const void* q_f16, const vo
     cudaError_t pe = cudaGetLastError();
     if (pe != cudaSuccess) return static_cast<int>(pe);
     if (umma) {
-        // the tcgen05 form of the step (decode_umma.cu), then the same merge
+        // the tcgen05 form of the step (decode_umma.cu); a step that has written its outputs gets no merge kernel
         rc = launch_decode_umma(R, prm, s);
         if (rc) return rc;
         return launch_merge<128>(prm, s);

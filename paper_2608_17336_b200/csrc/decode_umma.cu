@@ -55,8 +55,8 @@ constexpr int kOffSmall = kOffMeta + kMetaTiles * 8;
 static_assert(kOffRing % 1024 == 0 && kOffV16 % 1024 == 0, "swizzled tiles start on 1 KB boundaries");
 
 // Two independent softmax streams of four warps each: stream g takes the steps (pairs of key tiles) j = g, g + 2, ...
-// with its own running maximum, row sums and O accumulator, and ends as its own partial result -- to the merge
-// kernel a CTA is two splits.  A stream's step is a chain of waits and short dependent instruction runs
+// with its own running maximum, row sums and O accumulator, and ends as its own partial result -- to whatever
+// merges, a CTA is two splits.  A stream's step is a chain of waits and short dependent instruction runs
 // (~2600 clk); two of them in flight hide that latency.
 constexpr int kStreams = 2, kStreamWarps = 4, kSoftmaxWarps = kStreams * kStreamWarps, kConvWarps = 16;
 constexpr int kConvWarp0 = kSoftmaxWarps, kProducerWarp = kConvWarp0 + kConvWarps;
@@ -588,7 +588,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
         const uint32_t col_o = kColO + g * 128;
         const int64_t orow = out_row0 + static_cast<int64_t>(lane < R ? lane : 0) * n_parts + g;   // (lanes < R of quarter 0)
         if (g >= n_pairs) {
-            // a stream without a step: an empty partial result, which the merge skips
+            // a stream without a step: an empty partial result, which every merge (the one at the CTA's end too) skips
             for (int idx = key; !alone && idx < R * D; idx += kStreamWarps * 32)
                 prm.o_part[(out_row0 + static_cast<int64_t>(idx / D) * n_parts + g) * D + (idx % D)] = 0.f;
             if (wq == 0 && lane < R) {
@@ -714,7 +714,7 @@ decode_umma_kernel(const __grid_constant__ CUtensorMap tm_k8, const __grid_const
                 if (!wait(&sh.zbar[g], 0, kWXchg)) break;
                 if (!wait(&sh.pv_pair[g], par, kWPV)) break;      // the PVs of this step
                 ptx::tc_fence_after_sync();
-    #pragma unroll 1
+#pragma unroll 1
                 for (int c = 0; c < D / 32 && !alone; ++c) {
                     uint32_t o[32];
                     ptx::tmem_ld32(tmem_base + col_o + 32 * c, o);
