@@ -73,9 +73,12 @@ constexpr float kLn2 = 0.6931471805599453f;
 // account it is hardly ever one row's affair: kAccept is half of what FP16 holds, not less (at 2^8, 32 heads x 8K with
 // outlier channels took 628 us in place of 590; maps and inputs whose m rarely moves take the same time).
 // An INT8 value cache multiplies P by its block's scale before it is rounded, up to 65504 / 127 = 516 where the values were
-// FP16: kAcceptScaled keeps that product below 33 020.
-constexpr float kAccept = 32768.f, kAcceptScaled = 64.f, kMove = 4.0f, kMargin = 6.0f;
+// FP16: kAcceptScaled keeps that product below 33 020.  There m moves from kMoveScaled on, so that a rejected step moves it
+// as well: with kMove, keys whose scores stay 8 to 10 binades above the first ones had every step redone (2K chunk of 24K, 32 / 8
+// heads, such a plateau 1230 us, now 640; without one 638).
+constexpr float kAccept = 32768.f, kAcceptScaled = 64.f, kMove = 4.0f, kMoveScaled = 1.5f, kMargin = 6.0f;
 static_assert(kAcceptScaled * (65504.f / 127.f) < 65504.f, "scaled probabilities of an accepted step are finite in FP16");
+static_assert(kAccept / 16.f > 16.f && kMove <= 4.f && kAcceptScaled / 16.f >= 4.f && kMoveScaled < 2.f, "a rejected step moves m");
 
 enum Role : int { kRoleSoftmaxA = 0, kRoleSoftmaxB = 1, kRoleProducer = 2, kRoleMma = 3, kRoleQuant = 4 };
 enum Bar : int { kBarQ = 0, kBarRingFull = 1, kBarRingEmpty = 2, kBarS = 3, kBarP = 4, kBarO = 5, kBarDrain = 6, kBarPV = 7,
@@ -1079,7 +1082,7 @@ attention_kernel(const Params prm, const __grid_constant__ CUtensorMap tm_q16,
                     for (int k = 0; k < 2; ++k) {
                         // a > 0, so max(a*raw) = a*max(raw)
                         const float m_step = quad_max(KH ? fmaxf(mx_lo[k], mx[k] * a_hi) : mx[k] * a);
-                        if (m_step > m_run[k] + kMove) {
+                        if (m_step > m_run[k] + (VS ? kMoveScaled : kMove)) {
                             alpha[k] = fast_exp2(m_run[k] - (m_step + kMargin));
                             m_run[k] = m_step + kMargin;
                             z[k] *= alpha[k];

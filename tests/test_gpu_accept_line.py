@@ -132,3 +132,35 @@ def test_one_key_a_step_with_large_value_scales(d, half, Hq, Hk, climb):
         ref = _reference(q[0], k[0], vd, *(x[0] for x in codes), int8, d, blk_k)
         assert torch.isfinite(out).all()
         assert (out.double() - ref).abs().max() < (2.0 ** -10 + 2.0 ** -14) * vd.abs().amax(), int8
+
+
+@pytest.mark.parametrize("d,climb", [(128, 8.6), (128, 9.5), (64, 9.0)])
+def test_a_rejected_step_moves_the_maximum(d, climb):
+    """INT8 value cache, keys that stay `climb` binades above the first ones: 2^(climb - 6) a key is over the line of a step's
+    sums.  If m stayed where it is, every step would be redone; that took 1.9 times as long, and takes as long as without."""
+    from paper_2608_17336_b200 import binding as tm
+    Hq, Hk, L, ctx = 32, 8, 1024, 8192
+    gen = torch.Generator(device=DEV).manual_seed(d)
+    whole, p = tm.problem(1, Hk, Hk, ctx, d, d, d, 1), tm.problem(1, Hq, Hk, L, d, d, d, 1)
+    q, k, v = (0.1 * torch.randn(s, generator=gen, device=DEV) for s in ((1, Hq, L, d), (1, Hk, ctx, d), (1, Hk, ctx, d)))
+    q[..., 0], k[..., 0] = 8.0, 0.0
+    words, _ = tm.tilemix_pack_routing_mask(whole, torch.zeros((1, Hk, whole.T_m, whole.T_mask), dtype=torch.uint8, device=DEV))
+    q, v = q.half(), v.half()
+    _, v8, _, vs = tm.tilemix_quantize_qk(whole, v, v)
+    best = []
+    for height in (0.0, climb):
+        k[:, :, 128:, 0] = height * d ** 0.5 / (8.0 * 1.4426950408889634)
+        k16 = k.half()
+        q8, _, qs, _ = tm.tilemix_quantize_qk(p, q, k16[:, :, ctx - L:])
+        _, k8, _, ks = tm.tilemix_quantize_qk(whole, k16, k16)
+        times = []
+        for _ in range(8):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            for _ in range(4):
+                tm.tilemix_attention_fwd_chunk_v8(p, ctx, q, k16, v8, vs, q8, k8, qs, ks, words)
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        best.append(min(times))
+    assert best[1] < 1.4 * best[0], best
